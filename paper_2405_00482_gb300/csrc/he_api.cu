@@ -16,6 +16,8 @@ void encode_set_smem_limits(int max_bytes);
 void cdiag_set_smem_limits(int max_bytes);
 void bconv_set_smem_limits(int max_bytes);
 void keyswitch_set_smem_limits(int max_bytes);
+void cdiag_tc_set_smem_limits();
+int cdiag_tc_tables(he_ctx *ctx);
 
 namespace {
 
@@ -180,6 +182,7 @@ static int set_smem_limits_once() {
     cdiag_set_smem_limits(smem);
     bconv_set_smem_limits(smem);
     keyswitch_set_smem_limits(smem);
+    cdiag_tc_set_smem_limits();
     if (cudaGetLastError() != cudaSuccess) return HE_ECUDA;
     done[dev] = true;
     return HE_OK;
@@ -405,6 +408,11 @@ int he_ctx_create(const he_params *p, uint64_t seed, void *stream, he_ctx **out)
         }
         ctx->moddown.push_back(md);
     }
+    if (cudaHostAlloc(&ctx->sh->dev_err, sizeof(unsigned int), cudaHostAllocMapped) != cudaSuccess) {
+        he_ctx_destroy(ctx);
+        return HE_ENOMEM;
+    }
+    *ctx->sh->dev_err = 0;
     bool ok = cuda_ok(cudaMalloc(&ctx->d_mc, sizeof(ModConst) * LK)) && cuda_ok(cudaMalloc(&ctx->d_tw, tw.size() * 8)) &&
               cuda_ok(cudaMalloc(&ctx->d_fft, fft.size() * 4)) && cuda_ok(cudaMalloc(&ctx->d_sk, (size_t)LK * N * 8)) &&
               cuda_ok(cudaMalloc(&ctx->d_sk_mont, (size_t)LK * N * 8));
@@ -438,6 +446,7 @@ int he_ctx_create(const he_params *p, uint64_t seed, void *stream, he_ctx **out)
         return HE_ECUDA;
     }
     rc = bconv_i8_tables(ctx);
+    if (rc == HE_OK) rc = cdiag_tc_tables(ctx);
     if (rc != HE_OK) {
         he_ctx_destroy(ctx);
         return rc;
@@ -488,6 +497,7 @@ int he_ctx_fork(he_ctx *parent, void *stream, he_ctx **out) {
     ctx->ntt_form = parent->ntt_form;
     for (int f = 0; f < HE_NTT_FORMS; ++f) ctx->ntt_form_ms[f] = parent->ntt_form_ms[f];
     ctx->d_bconv_a = parent->d_bconv_a;
+    ctx->d_tc = parent->d_tc;
     ctx->bconv_a_off = parent->bconv_a_off;
     // the parent's pending work (keys, tables) must be complete before the fork's stream uses it
     if (cudaStreamSynchronize(parent->stream) != cudaSuccess) {
@@ -500,7 +510,8 @@ int he_ctx_fork(he_ctx *parent, void *stream, he_ctx **out) {
 
 int he_synchronize(he_ctx *ctx) {
     if (!ctx) return HE_EINVAL;
-    return he_check(cudaStreamSynchronize(ctx->stream));
+    const int rc = he_check(cudaStreamSynchronize(ctx->stream));
+    return rc == HE_OK && *ctx->sh->dev_err ? HE_ETIMEOUT : rc;
 }
 
 int he_launch_count(const he_ctx *ctx, int64_t *count) {

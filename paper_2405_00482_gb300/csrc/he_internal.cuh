@@ -138,10 +138,12 @@ struct he_shared {
     std::map<uint32_t, uint64_t *> keys;      // Galois element -> [dnum][2][L+K][N]
     int key_fusion = 1;                       // fused key tables of encoded matrices: 0 never, 1 on reuse, 2 always
     size_t fuse_max = (size_t)8 << 30;        // largest fused table built (bytes)
-    void *owned[6] = {};                      // device tables: d_mc, d_tw, d_fft, d_sk, d_sk_mont, d_bconv_a
+    void *owned[7] = {};                      // device tables: d_mc, d_tw, d_fft, d_sk, d_sk_mont, d_bconv_a, d_tc
+    unsigned int *dev_err = nullptr;          // page-locked: set by a kernel whose bounded wait gave up
     ~he_shared() {
         for (auto &kv : keys) cudaFree(kv.second);
         for (void *p : owned) cudaFree(p);
+        cudaFreeHost(dev_err);
     }
     uint64_t *key(uint32_t g) {
         std::lock_guard<std::mutex> lock(mu);
@@ -179,6 +181,7 @@ struct he_ctx {
     int ks_variant = -1;              // transform variant of the many-rotation key switch, chosen by timing (-1: not yet)
     float ks_tune_ms[HE_KS_VARIANTS] = {};  // the timed milliseconds of each variant (one full chunk of rotations)
     uint32_t *d_bconv_a = nullptr;    // INT8 engine: tensor-core A fragments of every (level, digit), shared with forks
+    void *d_tc = nullptr;             // tensor-core product of Alg. 3: reconstruction constants per prime (he_cdiag_tc.cu)
     std::vector<size_t> bconv_a_off;  // their offsets (uint4 units), [level * dnum + digit]
     // staging of the host-memory entry points (he_host.cu), grown on demand: a device buffer for
     // inputs and results, a page-locked host buffer for copies from or to pageable memory, and
