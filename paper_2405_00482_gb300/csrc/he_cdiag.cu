@@ -156,6 +156,44 @@ __global__ void cdiag_rescale_kernel(const uint64_t *__restrict__ pre, const uin
     for (int x = threadIdx.x; x < N; x += blockDim.x) o[x] = mul_shoup(sub_mod(cj[x], s[SIDX(x)], q), rc.inv[j], rc.inv_shoup[j], q);
 }
 
+// The same in two phases of small CTAs (he_ntt.cuh, NTT form 2; log N = 12..14): the columns on the
+// centred last limb into the output, then the rows with the combination as their store.
+template <int LOGN>
+__global__ void __launch_bounds__(NTT2_THREADS, 8) cdiag_rescale_cols_kernel(const uint64_t *__restrict__ last, int level, uint64_t ql,
+                                                                           const __grid_constant__ OutTable outs, int k_first,
+                                                                           const uint64_t *__restrict__ d_tw, const ModConst *__restrict__ mc) {
+    HE_GRID_DEP();
+    constexpr int N = 1 << LOGN, TILES = (N >> 6) / NTT2_TC;
+    __shared__ uint64_t sm[ntt2_cols_smem_words()];
+    const int item = blockIdx.x / TILES, c0 = (blockIdx.x % TILES) * NTT2_TC;
+    const int kl = item / (2 * level), c = (item / level) % 2, j = item % level;
+    const uint64_t q = mc[j].q, mu = mc[j].mu, half = ql / 2;
+    const uint64_t *lc = last + ((int64_t)(k_first + kl) * 2 + c) * N;
+    ntt2_fwd_cols<LOGN>(
+        sm,
+        [=](int64_t x) {
+            uint64_t r = lc[x] + half;
+            if (r >= ql) r -= ql;
+            return reduce_signed((int64_t)r - (int64_t)half, q, mu);
+        },
+        outs.p[kl] + ((int64_t)c * level + j) * N, c0, TwGlobal{twiddles(d_tw, j, 0, LOGN)}, q);
+}
+template <int LOGN>
+__global__ void __launch_bounds__(NTT2_THREADS, 8) cdiag_rescale_rows_kernel(const uint64_t *__restrict__ pre, int level, const __grid_constant__ CdRescale rc,
+                                                                           const __grid_constant__ OutTable outs, int k_first,
+                                                                           const uint64_t *__restrict__ d_tw, const ModConst *__restrict__ mc) {
+    HE_GRID_DEP();
+    constexpr int N = 1 << LOGN, TILES = 64 / NTT2_TR;
+    __shared__ uint64_t sm[ntt2_frows_smem_words(LOGN - 6)];
+    const int item = blockIdx.x / TILES, b0 = (blockIdx.x % TILES) * NTT2_TR;
+    const int kl = item / (2 * level), c = (item / level) % 2, j = item % level;
+    const uint64_t q = mc[j].q, inv = rc.inv[j], invs = rc.inv_shoup[j];
+    const uint64_t *cj = pre + (((int64_t)(k_first + kl) * 2 + c) * (level + 1) + j) * N;
+    uint64_t *o = outs.p[kl] + ((int64_t)c * level + j) * N;
+    ntt2_fwd_rows<LOGN>(sm, o, b0, TwGlobal{twiddles(d_tw, j, 0, LOGN)}, q, mc[j].mu,
+                        [=](int x, uint64_t v) { o[x] = mul_shoup(sub_mod(cj[x], v, q), inv, invs, q); });
+}
+
 // slots of the diagonals e_i[j] = A[j mod m, (i + j) mod n], repeated over the N/2 slots
 __global__ void cdiag_layout_kernel(const double *__restrict__ A, int64_t m, int64_t n, int64_t slots, double *out) {
     HE_GRID_DEP();
@@ -269,11 +307,15 @@ int he_cdiag_encode_matrix(he_ctx *ctx, const double *A, int64_t m, int64_t n, d
     ctx->launches++;
     launch_k(cdiag_layout_kernel, blocks_for(lo * (N / 2)), 256, 0, ctx->stream, A, m, n, N / 2, slots);
     launch_encode(ctx, slots, N / 2, N / 2, (int)lo, scale, coef);
+    // every diagonal's transforms in one pair of launches: one launch per diagonal (7 limb-polys on 8-CTA
+    // clusters at N = 2^14) took 10.9 us each, 2.8 ms for 256, with most SMs idle
+    std::vector<uint64_t *> ptrs((size_t)lo);
     for (int64_t i = 0; i < lo; ++i) {
-        launch_ntt_from_int64(ctx, coef + i * N, outs[i].data, 1, map, 0);
+        ptrs[(size_t)i] = outs[i].data;
         outs[i].level = level;
         outs[i].scale = scale;
     }
+    launch_ntt_from_int64_tab(ctx, coef, ptrs.data(), (int)lo, map);
     return cudaGetLastError() == cudaSuccess ? HE_OK : HE_ECUDA;
 }
 
@@ -324,6 +366,19 @@ int he_cdiag_matmult(he_ctx *ctx, const he_cdmat *W, const he_ct *cts, int n_ct,
         const int kn = (int)std::min<int64_t>(CD_MAX_OUT, K - kf);
         OutTable ot;
         for (int k = 0; k < kn; ++k) ot.p[k] = outs[kf + k].data;
+        if (use_two_phase(ctx, kn * 2 * level)) {
+            const unsigned cols = (unsigned)(kn * 2 * level * ((N >> 6) / NTT2_TC)), rows = (unsigned)(kn * 2 * level * (64 / NTT2_TR));
+            auto go = [&](auto L) {
+                launch_k(cdiag_rescale_cols_kernel<decltype(L)::value>, cols, NTT2_THREADS, 0, ctx->stream, last, level, rc.ql, ot, (int)kf, ctx->d_tw,
+                         ctx->d_mc);
+                launch_k(cdiag_rescale_rows_kernel<decltype(L)::value>, rows, NTT2_THREADS, 0, ctx->stream, pre, level, rc, ot, (int)kf, ctx->d_tw, ctx->d_mc);
+            };
+            if (ctx->log_n == 12) go(std::integral_constant<int, 12>{});
+            else if (ctx->log_n == 13) go(std::integral_constant<int, 13>{});
+            else go(std::integral_constant<int, 14>{});
+            ctx->launches += 2;
+            continue;
+        }
         ctx->launches++;
         launch_k(cdiag_rescale_kernel, kn * 2 * level, ntt_threads(ctx->log_n), ntt_smem_bytes(ctx->log_n), ctx->stream, pre, last, level, rc, ot, (int)kf, ctx->d_tw, ctx->d_mc, ctx->log_n);
     }

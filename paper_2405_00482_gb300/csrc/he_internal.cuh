@@ -425,6 +425,8 @@ size_t cl_smem_bytes(int logn);
 inline size_t ntt_smem_bytes(int logn) { return ((size_t)1 << logn) * 8 + ((size_t)1 << logn) / 32 * 8; }
 // NTT forward of signed int64 coefficient vectors reduced per limb: in [groups][N] -> out [groups][map.n][N]
 void launch_ntt_from_int64(he_ctx *ctx, const int64_t *in, uint64_t *out, int groups, const LimbMap &map, int to_mont);
+// the same with group g's output at outs[g], the groups in one pair of launches (log N = 12..14)
+void launch_ntt_from_int64_tab(he_ctx *ctx, const int64_t *in, uint64_t *const *outs, int groups, const LimbMap &map);
 // x -> x 2^64 mod q in place
 void launch_to_mont(he_ctx *ctx, uint64_t *data, int groups, const LimbMap &map);
 

@@ -11,6 +11,11 @@
 
 namespace {
 
+#define HE_OUT_PTRS 256  // output pointers passed by value to one launch
+struct OutPtrs {
+    uint64_t *p[HE_OUT_PTRS];
+};
+
 // LOGN > 0: the ring size at compile time (logn_rt == LOGN); 0: at run time
 template <bool CL, int LOGN = 0>
 __global__ void ntt_fwd_kernel(const uint64_t *__restrict__ in, int64_t in_gs, uint64_t *out, int64_t out_gs, LimbMap map,
@@ -174,6 +179,30 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) ntt2_cols_kernel(const void *
     }
 }
 
+// the same two phases with each group's output at a pointer of its own ([map.n][N] each)
+template <int LOGN>
+__global__ void __launch_bounds__(NTT2_THREADS, 8) ntt2_cols_tab_kernel(const int64_t *__restrict__ in, const __grid_constant__ OutPtrs outs, LimbMap map,
+                                                                      const uint64_t *__restrict__ d_tw, const ModConst *__restrict__ mc) {
+    HE_GRID_DEP();
+    constexpr int N = 1 << LOGN, TILES = (N >> 6) / NTT2_TC;
+    __shared__ uint64_t sm[ntt2_cols_smem_words()];
+    const int poly = blockIdx.x / TILES, c0 = (blockIdx.x % TILES) * NTT2_TC;
+    const int g = poly / map.n, l = poly % map.n, p = map.prime[l];
+    const uint64_t q = mc[p].q, mu = mc[p].mu;
+    const int64_t *src = in + (int64_t)g * N;
+    ntt2_fwd_cols<LOGN>(sm, [=](int64_t x) { return reduce_signed(src[x], q, mu); }, outs.p[g] + (int64_t)l * N, c0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, q);
+}
+template <int LOGN>
+__global__ void __launch_bounds__(NTT2_THREADS, 8) ntt2_rows_tab_kernel(const __grid_constant__ OutPtrs outs, LimbMap map, const uint64_t *__restrict__ d_tw,
+                                                                      const ModConst *__restrict__ mc) {
+    HE_GRID_DEP();
+    constexpr int N = 1 << LOGN, TILES = 64 / NTT2_TR;
+    __shared__ uint64_t sm[ntt2_frows_smem_words(LOGN - 6)];
+    const int poly = blockIdx.x / TILES, b0 = (blockIdx.x % TILES) * NTT2_TR;
+    const int g = poly / map.n, l = poly % map.n, p = map.prime[l];
+    ntt2_fwd_rows<LOGN>(sm, outs.p[g] + (int64_t)l * N, b0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, mc[p].q, mc[p].mu);
+}
+
 template <int LOGN>
 __global__ void __launch_bounds__(NTT2_THREADS, 8) ntt2_rows_kernel(uint64_t *data, int64_t gs, LimbMap map, const uint64_t *__restrict__ d_tw,
                                                                   const ModConst *__restrict__ mc) {
@@ -266,7 +295,7 @@ static auto pair_instance(int logn, F f) {
 
 bool use_pair(const he_ctx *ctx, int polys) { return ctx->ntt_form == 1 && !use_cluster(ctx->log_n, polys) && ctx->log_n >= 12 && ctx->log_n <= 14; }
 bool use_two_phase(const he_ctx *ctx, int polys) {
-    return ctx->ntt_form == 2 && !use_cluster(ctx->log_n, polys) && ctx->log_n >= 12 && ctx->log_n <= 14;
+    return (ctx->ntt_form == 2 || ctx->ntt_form < 0) && !use_cluster(ctx->log_n, polys) && ctx->log_n >= 12 && ctx->log_n <= 14;
 }
 
 // the two launches of the two-phase forward transform (from int64 coefficients when I64)
@@ -382,6 +411,30 @@ void launch_ntt_from_int64(he_ctx *ctx, const int64_t *in, uint64_t *out, int gr
         // kernels find room beside it (capping it at two per SM made the encoded matrix alone
         // faster, 80 against 95 us, and the benchmark step 3% slower)
         launch_k(k, polys, ntt_threads(ctx->log_n), ntt_smem_bytes(ctx->log_n), ctx->stream, in, out, map, ctx->d_tw, ctx->d_mc, ctx->log_n, to_mont);
+    }
+}
+
+void launch_ntt_from_int64_tab(he_ctx *ctx, const int64_t *in, uint64_t *const *outs, int groups, const LimbMap &map) {
+    if (ctx->log_n < 12 || ctx->log_n > 14 || use_cluster(ctx->log_n, groups * map.n)) {
+        for (int g = 0; g < groups; ++g) launch_ntt_from_int64(ctx, in + (int64_t)g * ctx->n, outs[g], 1, map, 0);
+        return;
+    }
+    const uint64_t *tw = ctx->d_tw;
+    const ModConst *mc = ctx->d_mc;
+    for (int g0 = 0; g0 < groups; g0 += HE_OUT_PTRS) {
+        const int n = std::min(HE_OUT_PTRS, groups - g0), polys = n * map.n;
+        OutPtrs tab{};
+        for (int g = 0; g < n; ++g) tab.p[g] = outs[g0 + g];
+        const int64_t *src = in + (int64_t)g0 * ctx->n;
+        const unsigned cols = (unsigned)(polys * ((ctx->n >> 6) / NTT2_TC)), rows = (unsigned)(polys * (64 / NTT2_TR));
+        auto go = [&](auto L) {
+            launch_k(ntt2_cols_tab_kernel<decltype(L)::value>, cols, NTT2_THREADS, 0, ctx->stream, src, tab, map, tw, mc);
+            launch_k(ntt2_rows_tab_kernel<decltype(L)::value>, rows, NTT2_THREADS, 0, ctx->stream, tab, map, tw, mc);
+        };
+        if (ctx->log_n == 12) go(std::integral_constant<int, 12>{});
+        else if (ctx->log_n == 13) go(std::integral_constant<int, 13>{});
+        else go(std::integral_constant<int, 14>{});
+        ctx->launches += 2;
     }
 }
 

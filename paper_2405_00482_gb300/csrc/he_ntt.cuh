@@ -414,9 +414,10 @@ __device__ __forceinline__ void ntt2_fwd_cols(uint64_t *sm, LOAD load, uint64_t 
 // canonical outputs.  The rows are staged into shared memory (sm: ntt2_rows_smem_words) as the
 // slice [b0 R, (b0 + NTT2_TR) R) of the transform and run through the one-CTA form's passes of up
 // to three stages (ntt_fwd_pass over the sets whose elements fall in the slice, as a cluster
-// member does), so a thread holds 8 values at a time.
-template <int LOGN>
-__device__ __forceinline__ void ntt2_fwd_rows(uint64_t *sm, uint64_t *poly, int b0, TwGlobal tw, uint64_t q, uint64_t mu) {
+// member does), so a thread holds 8 values at a time.  Element x's canonical result v goes to
+// store(x, v) (the form without it writes it back in place).
+template <int LOGN, class STORE>
+__device__ __forceinline__ void ntt2_fwd_rows(uint64_t *sm, const uint64_t *poly, int b0, TwGlobal tw, uint64_t q, uint64_t mu, STORE store) {
     constexpr int LB = LOGN - 6, R = 1 << LB, LEN = NTT2_TR * R;
     const int off = b0 * R;  // a multiple of 32, so SIDX splits over the offset
     stage_in(sm, poly + off, LEN, [](uint64_t v) { return v; });
@@ -448,8 +449,12 @@ __device__ __forceinline__ void ntt2_fwd_rows(uint64_t *sm, uint64_t *poly, int 
     // without the lazy correction the values are below (1 + 2 log N) q: one Barrett step
     for (int k = threadIdx.x; k < LEN; k += NTT2_THREADS) {
         const uint64_t v = sm[SIDX(k)];
-        poly[off + k] = corr ? v : reduce_barrett(v, q, mu);
+        store(off + k, corr ? v : reduce_barrett(v, q, mu));
     }
+}
+template <int LOGN>
+__device__ __forceinline__ void ntt2_fwd_rows(uint64_t *sm, uint64_t *poly, int b0, TwGlobal tw, uint64_t q, uint64_t mu) {
+    ntt2_fwd_rows<LOGN>(sm, poly, b0, tw, q, mu, [=](int x, uint64_t v) { poly[x] = v; });
 }
 
 // inverse stages 0 .. log N - 7 of rows b0 .. b0 + NTT2_TR - 1 of one limb-poly (inputs below 2q),
