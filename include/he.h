@@ -165,7 +165,7 @@ int he_rotate(he_ctx *ctx, const he_ct *in, int32_t step, he_ct *out);
 int he_rotate_hoisted(he_ctx *ctx, const he_ct *in, const int32_t *steps, int k, he_ct *outs);
 /* O3 on many different ciphertexts, each by its own step (outs[i] = RotL(ins[i], steps[i]),
  * bit-identical to he_rotate per pair), as one launch per stage over all of them (in chunks of
- * 64): ModUp, key-switch inner product, ModDown.  All inputs at one level; outputs must not
+ * 128): ModUp, key-switch inner product, ModDown.  All inputs at one level; outputs must not
  * overlap any input (HE_EINVAL); a missing Galois key gives HE_EKEY; steps that are multiples
  * of N/2 copy. */
 int he_rotate_many(he_ctx *ctx, const he_ct *ins, const int32_t *steps, int count, he_ct *outs);
@@ -253,7 +253,7 @@ int he_matmult_plain_cipher_noalloc(he_ctx *ctx, const he_plan *plan, const he_p
  * runs its transforms as one CTA per limb-poly with the usual thread count (variant 0), with
  * 512 threads and at most 64 registers (variant 1), or in two phases of small CTAs per transform
  * (variant 2, log N = 12..14: the NTT form 2 split into rows and columns, see he_ntt_form).  The
- * first such call on a context times them on its first chunk (synchronising the stream; not
+ * first such call on a context times them on its first 32 rotations (synchronising the stream; not
  * under stream capture) and keeps the fastest: variant (-1 before) and ms[0..HE_KS_VARIANTS-1]
  * (may be NULL) report the choice and the timings.  Every variant gives the same residues. */
 #define HE_KS_VARIANTS 3

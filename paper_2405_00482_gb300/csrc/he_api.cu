@@ -367,6 +367,8 @@ int he_ctx_create(const he_params *p, uint64_t seed, void *stream, he_ctx **out)
                     if (j != i) hat_qi = hmul(hat_qi, ctx->primes[j] % qi, qi);
                 mu.inv[d][i - lo] = hinv(hat_qi, qi);
                 mu.inv_shoup[d][i - lo] = shoup(mu.inv[d][i - lo], qi);
+                mu.ninv_inv[i] = hmul(ctx->mc[i].ninv, mu.inv[d][i - lo], qi);
+                mu.ninv_inv_shoup[i] = shoup(mu.ninv_inv[i], qi);
                 for (int u = 0; u < mu.ext; ++u) {
                     const uint64_t t = ctx->primes[mu.ext_prime[u]];
                     uint64_t h = 1 % t;
@@ -390,6 +392,8 @@ int he_ctx_create(const he_params *p, uint64_t seed, void *stream, he_ctx **out)
                 if (r != i) hat = hmul(hat, ctx->primes[ctx->L + r] % pi, pi);
             md.inv[i] = hinv(hat, pi);
             md.inv_shoup[i] = shoup(md.inv[i], pi);
+            md.ninv_inv[i] = hmul(ctx->mc[ctx->L + i].ninv, md.inv[i], pi);
+            md.ninv_inv_shoup[i] = shoup(md.ninv_inv[i], pi);
             for (int j = 0; j <= level; ++j) {
                 const uint64_t q = ctx->primes[j];
                 uint64_t h = 1 % q;

@@ -47,6 +47,15 @@ __device__ __forceinline__ uint64_t mul_shoup_lazy(uint64_t x, uint64_t w, uint6
     return x * w - __umul64hi(x, wp) * q;
 }
 
+// sum_i x_i h_i as a transform's input: the lazy Shoup products (each below 2q, for any x_i < 2^64) of
+// up to four terms, brought below 4q (Harvey's bound on a forward butterfly's inputs)
+template <class X>
+__device__ __forceinline__ uint64_t conv_lazy(int n, X x, const uint64_t *h, const uint64_t *hs, int stride, uint64_t q) {
+    uint64_t a = mul_shoup_lazy(x(0), h[0], hs[0], q);
+    for (int i = 1; i < n; ++i) a += mul_shoup_lazy(x(i), h[i * stride], hs[i * stride], q);
+    return n > 2 && a >= 4 * q ? a - 4 * q : a;
+}
+
 // Montgomery reduction of T = hi 2^64 + lo < q 2^64: returns T 2^-64 mod q in [0, q).
 // qinv = -q^-1 mod 2^64.
 __device__ __forceinline__ uint64_t redc(uint64_t hi, uint64_t lo, uint64_t q, uint64_t qinv) {
@@ -119,6 +128,8 @@ struct ModUpConst {
     uint64_t inv[HE_MAX_DNUM][4], inv_shoup[HE_MAX_DNUM][4];
     // (Qd/q_i) mod target prime of extended limb u, with Shoup companion
     uint64_t hat[HE_MAX_DNUM][4][HE_MAX_LIMBS], hat_shoup[HE_MAX_DNUM][4][HE_MAX_LIMBS];
+    // N^-1 (Qd/q_l)^-1 mod q_l of limb l in its digit: the inverse transform's factor with inv folded in
+    uint64_t ninv_inv[HE_MAX_Q], ninv_inv_shoup[HE_MAX_Q];
 };
 
 // constants for ModDown of one level (Q_level U P -> Q_level)
@@ -129,6 +140,7 @@ struct ModDownConst {
     uint64_t inv[HE_MAX_P], inv_shoup[HE_MAX_P];                      // [(P/p_i)^-1]_{p_i}
     uint64_t hat[HE_MAX_P][HE_MAX_Q], hat_shoup[HE_MAX_P][HE_MAX_Q];  // (P/p_i) mod q_j
     uint64_t pinv[HE_MAX_Q], pinv_shoup[HE_MAX_Q];                    // P^-1 mod q_j
+    uint64_t ninv_inv[HE_MAX_P], ninv_inv_shoup[HE_MAX_P];            // N^-1 [(P/p_i)^-1]_{p_i}
 };
 
 // What the contexts of one family (a context and its forks) share: the device tables, the
@@ -179,7 +191,7 @@ struct he_ctx {
                                       // (forward only; -1: not yet timed)
     float ntt_form_ms[HE_NTT_FORMS] = {};  // the timed milliseconds of each form (an encoded matrix's transform)
     int ks_variant = -1;              // transform variant of the many-rotation key switch, chosen by timing (-1: not yet)
-    float ks_tune_ms[HE_KS_VARIANTS] = {};  // the timed milliseconds of each variant (one full chunk of rotations)
+    float ks_tune_ms[HE_KS_VARIANTS] = {};  // the timed milliseconds of each variant (the first 32 rotations)
     uint32_t *d_bconv_a = nullptr;    // INT8 engine: tensor-core A fragments of every (level, digit), shared with forks
     void *d_tc = nullptr;             // tensor-core product of Alg. 3: reconstruction constants per prime (he_cdiag_tc.cu)
     std::vector<size_t> bconv_a_off;  // their offsets (uint4 units), [level * dnum + digit]
@@ -242,7 +254,7 @@ struct RotJob {
 };
 // up to HE_ROT_CHUNK rotations, passed to the kernels by value (kernel parameters), so a launch
 // needs no copy of a job table to the device
-#define HE_ROT_CHUNK 64
+#define HE_ROT_CHUNK 128
 struct RotTable {
     RotJob j[HE_ROT_CHUNK];
 };

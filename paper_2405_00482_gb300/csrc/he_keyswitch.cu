@@ -117,8 +117,8 @@ __global__ void ks_p_kernel(const RotTable jobs, KsGeom kg, ModDownConst md, con
     __syncthreads();
     inv_any<CL, LOGN>(s, itw, q, logn);
     uint64_t *dst = kg.pc + (((int64_t)j * 2 + c) * kg.K + i) * N + off;
-    const uint64_t ni = mc[pr].ninv, nis = mc[pr].ninv_shoup;
-    for (int k = threadIdx.x; k < len; k += B) dst[k] = mul_shoup(mul_shoup(s[SIDX(k)], ni, nis, q), md.inv[i], md.inv_shoup[i], q);
+    const uint64_t f = md.ninv_inv[i], fs = md.ninv_inv_shoup[i];
+    for (int k = threadIdx.x; k < len; k += B) dst[k] = mul_shoup(s[SIDX(k)], f, fs, q);
 }
 
 template <bool CL, int LOGN, int ND>
@@ -237,8 +237,8 @@ __global__ void __launch_bounds__(512, TPB == 512 ? 2 : 1) ks_pintt_kernel(KsGeo
     stage_in(s, x, len, [](uint64_t v) { return v; });
     __syncthreads();
     inv_any<CL, LOGN>(s, itw, q, logn);
-    const uint64_t ni = mc[pr].ninv, nis = mc[pr].ninv_shoup;
-    for (int k = threadIdx.x; k < len; k += blockDim.x) x[k] = mul_shoup(mul_shoup(s[SIDX(k)], ni, nis, q), md.inv[i], md.inv_shoup[i], q);
+    const uint64_t f = md.ninv_inv[i], fs = md.ninv_inv_shoup[i];
+    for (int k = threadIdx.x; k < len; k += blockDim.x) x[k] = mul_shoup(s[SIDX(k)], f, fs, q);
 }
 
 // item (j, c, l): cv_j[c][l] = NTT(sum_i pc_j[c][i] (P/p_i mod q_l))
@@ -287,33 +287,34 @@ __global__ void __launch_bounds__(NTT2_THREADS) ks2_pinv_rows_kernel(KsGeom kg, 
 }
 
 template <int LOGN>
-__global__ void __launch_bounds__(NTT2_THREADS, 8) ks2_pinv_cols_kernel(KsGeom kg, ModDownConst md, const uint64_t *__restrict__ d_tw,
+__global__ void __launch_bounds__(NTT2_THREADS, 8) ks2_pinv_cols_kernel(KsGeom kg, const __grid_constant__ ModDownConst md, const uint64_t *__restrict__ d_tw,
                                                                       const ModConst *__restrict__ mc) {
     HE_GRID_DEP();
     constexpr int N = 1 << LOGN, TILES = (N >> 6) / NTT2_TC;
     __shared__ uint64_t sm[ntt2_cols_smem_words()];
     const int item = blockIdx.x / TILES, c0 = (blockIdx.x % TILES) * NTT2_TC;
     const int i = item % kg.K, pr = md.p_prime[i];
-    const uint64_t q = mc[pr].q, ni = mc[pr].ninv, nis = mc[pr].ninv_shoup, f = md.inv[i], fs = md.inv_shoup[i];
+    const uint64_t q = mc[pr].q, f = md.ninv_inv[i], fs = md.ninv_inv_shoup[i];
     uint64_t *x = kg.pc + (int64_t)item * N;
     ntt2_inv_cols<LOGN>(sm, x, c0, TwGlobal{twiddles(d_tw, pr, 1, LOGN)}, q,
-                        [=](int64_t k, uint64_t v) { x[k] = mul_shoup(mul_shoup(v, ni, nis, q), f, fs, q); });
+                        [=](int64_t k, uint64_t v) { x[k] = mul_shoup(v, f, fs, q); });
 }
 
 template <int LOGN>
-__global__ void __launch_bounds__(NTT2_THREADS, 8) ks2_conv_cols_kernel(KsGeom kg, uint64_t *cv, ModDownConst md, const uint64_t *__restrict__ d_tw,
+__global__ void __launch_bounds__(NTT2_THREADS, 8) ks2_conv_cols_kernel(KsGeom kg, uint64_t *cv, const __grid_constant__ ModDownConst md, const uint64_t *__restrict__ d_tw,
                                                                       const ModConst *__restrict__ mc) {
     HE_GRID_DEP();
     constexpr int N = 1 << LOGN, TILES = (N >> 6) / NTT2_TC;
     __shared__ uint64_t sm[ntt2_cols_smem_words()];
     const int item = blockIdx.x / TILES, c0 = (blockIdx.x % TILES) * NTT2_TC;
     const int jc = item / kg.nl, l = item % kg.nl, pl = md.q_prime[l];
-    const uint64_t q = mc[pl].q, h0 = md.hat[0][l], h0s = md.hat_shoup[0][l];
+    const uint64_t q = mc[pl].q;
     const uint64_t *pc = kg.pc + (int64_t)jc * kg.K * N;
     ntt2_fwd_cols<LOGN>(
         sm,
         [&](int64_t x) {
-            uint64_t v = mul_shoup(pc[x], h0, h0s, q);
+            if (kg.K <= 4) return conv_lazy(kg.K, [&](int i) { return pc[(int64_t)i * N + x]; }, &md.hat[0][l], &md.hat_shoup[0][l], HE_MAX_Q, q);
+            uint64_t v = mul_shoup(pc[x], md.hat[0][l], md.hat_shoup[0][l], q);
             for (int i = 1; i < kg.K; ++i) v = add_mod(v, mul_shoup(pc[(int64_t)i * N + x], md.hat[i][l], md.hat_shoup[i][l], q), q);
             return v;
         },
@@ -407,9 +408,9 @@ void launch_keyswitch_many(he_ctx *ctx, const RotJob *jobs, int count, int level
     const int cmax = count < HE_ROT_CHUNK ? count : HE_ROT_CHUNK;
     uint64_t *cv = pc + (size_t)cmax * 2 * ctx->K * ctx->n;  // [cmax][2][level+1][N] after pc [cmax][2][K][N]
     // one chunk's launches with transform variant v (0: ntt_threads per CTA, 1: 512 threads,
-    // 2: two phases of small CTAs per transform)
-    auto issue = [&](int c0, int v) {
-        const int n = count - c0 < HE_ROT_CHUNK ? count - c0 : HE_ROT_CHUNK;
+    // 2: two phases of small CTAs per transform), of at most nmax rotations
+    auto issue = [&](int c0, int v, int nmax = HE_ROT_CHUNK) {
+        const int n = count - c0 < nmax ? count - c0 : nmax;
         RotTable tab{};
         for (int j = 0; j < n; ++j) tab.j[j] = jobs[c0 + j];
         KsGeom kg{};
@@ -479,7 +480,7 @@ void launch_keyswitch_many(he_ctx *ctx, const RotJob *jobs, int count, int level
         if (pe2) cudaEventRecord(pe2[1], st);
     };
     // the first launch of at least 32 rotations on a context chooses the transform variant by timing
-    // both on its first chunk (the launches overwrite their outputs with the same values, so
+    // each on its first 32 (the launches overwrite their outputs with the same values, so
     // repeating them changes nothing); not under stream capture, where the usual thread count is taken
     if (ctx->ks_variant < 0 && cmax >= 32 && !use_cluster(logn, cmax * 2 * (level + 1))) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -491,7 +492,7 @@ void launch_keyswitch_many(he_ctx *ctx, const RotJob *jobs, int count, int level
                 float ms = 1e30f;
                 for (int rep = 0; rep < 3; ++rep) {
                     cudaEventRecord(e0, st);
-                    issue(0, v);
+                    issue(0, v, 32);
                     cudaEventRecord(e1, st);
                     if (cudaEventSynchronize(e1) != cudaSuccess) break;
                     float t = 0.0f;

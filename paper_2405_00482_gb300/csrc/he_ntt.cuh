@@ -97,7 +97,7 @@ struct TwFirstInv {
 // at stage s0 + j element k meets twiddle entry m + (g << j) + (k >> (NB - j)), m = 2^(s0+j),
 // the 2^j consecutive entries loaded once per stage.  Harvey's lazy butterfly: inputs below 4q,
 // outputs below 4q.  Without CORR the top input is not brought below 2q first: each stage then
-// adds less than 2q to the bound, so canonical inputs stay below (1 + 2 log N) q, which fits in
+// adds less than 2q to the bound, so inputs below 4q stay below (4 + 2 log N) q, which fits in
 // 64 bits for q < 2^59 and log N <= 14 (the caller reduces at the end).
 template <int NB, class TWA, bool CORR = true>
 __device__ __forceinline__ void ntt_fwd_radix(uint64_t (&r)[1 << NB], TWA tw, uint64_t q, int s0, int g) {
@@ -385,7 +385,7 @@ __device__ __forceinline__ uint64_t signed_to_mont(int64_t v, uint64_t r1, uint6
 }
 
 // forward stages 0-5 of columns c0 .. c0 + NTT2_TC - 1 of one limb-poly: load(x) gives the
-// canonical input of element x; writes the stage-5 values to dst[x]
+// input of element x, below 4q; writes the stage-5 values to dst[x]
 template <int LOGN, class LOAD>
 __device__ __forceinline__ void ntt2_fwd_cols(uint64_t *sm, LOAD load, uint64_t *dst, int c0, TwGlobal tw, uint64_t q) {
     constexpr int C = (1 << LOGN) >> 6, PAD = NTT2_TC + 1;
@@ -446,7 +446,7 @@ __device__ __forceinline__ void ntt2_fwd_rows(uint64_t *sm, const uint64_t *poly
             else ntt_fwd_pass<1, TwGlobal, false>(sm, tw, q, LOGN, s0, false, off >> 1, (off + LEN) >> 1, off);
         }
     }
-    // without the lazy correction the values are below (1 + 2 log N) q: one Barrett step
+    // without the lazy correction the values are below (4 + 2 log N) q: one Barrett step
     for (int k = threadIdx.x; k < LEN; k += NTT2_THREADS) {
         const uint64_t v = sm[SIDX(k)];
         store(off + k, corr ? v : reduce_barrett(v, q, mu));

@@ -542,7 +542,7 @@ __global__ void rot_modup_kernel(const RotTable jobs, RotGeom rg, ModUpConst mu,
 }
 
 // ---- the same ModUp in two phases per transform (NTT form 2, he_ntt.cuh): the inverse NTT of
-// every c1 limb as rows (from the job's ciphertext into coef) then columns scaled by N^-1, and
+// every c1 limb as rows (from the job's ciphertext into coef) then columns scaled by N^-1 (Qd/q_i)^-1, and
 // every (j, d, u) target as columns on the conversion then rows; the digit's own limbs are
 // copied from the NTT-form input by the column launch and skipped by the row launch.  The values
 // of rot_intt_c1_kernel and rot_modup_kernel. ----
@@ -559,19 +559,19 @@ __global__ void __launch_bounds__(NTT2_THREADS) rot2_intt_rows_kernel(const RotT
 }
 
 template <int LOGN>
-__global__ void __launch_bounds__(NTT2_THREADS, 8) rot2_intt_cols_kernel(RotGeom rg, const uint64_t *__restrict__ d_tw, const ModConst *__restrict__ mc) {
+__global__ void __launch_bounds__(NTT2_THREADS, 8) rot2_intt_cols_kernel(RotGeom rg, const __grid_constant__ ModUpConst mu, const uint64_t *__restrict__ d_tw, const ModConst *__restrict__ mc) {
     HE_GRID_DEP();
     constexpr int N = 1 << LOGN, TILES = (N >> 6) / NTT2_TC;
     __shared__ uint64_t sm[ntt2_cols_smem_words()];
     const int item = blockIdx.x / TILES, c0 = (blockIdx.x % TILES) * NTT2_TC;
     const int j = item / rg.nl, l = item % rg.nl;
-    const uint64_t q = mc[l].q, ni = mc[l].ninv, nis = mc[l].ninv_shoup;
+    const uint64_t q = mc[l].q, ni = mu.ninv_inv[l], nis = mu.ninv_inv_shoup[l];
     uint64_t *x = rg.coef + j * rg.coef_w + (int64_t)l * N;
     ntt2_inv_cols<LOGN>(sm, x, c0, TwGlobal{twiddles(d_tw, l, 1, LOGN)}, q, [=](int64_t k, uint64_t v) { x[k] = mul_shoup(v, ni, nis, q); });
 }
 
 template <int LOGN>
-__global__ void __launch_bounds__(NTT2_THREADS, 8) rot2_modup_cols_kernel(const RotTable jobs, RotGeom rg, ModUpConst mu,
+__global__ void __launch_bounds__(NTT2_THREADS, 8) rot2_modup_cols_kernel(const __grid_constant__ RotTable jobs, RotGeom rg, const __grid_constant__ ModUpConst mu,
                                                                         const uint64_t *__restrict__ d_tw, const ModConst *__restrict__ mc) {
     HE_GRID_DEP();
     constexpr int N = 1 << LOGN, C = N >> 6, TILES = C / NTT2_TC;
@@ -591,19 +591,11 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) rot2_modup_cols_kernel(const 
         return;
     }
     const uint64_t *coef = rg.coef + j * rg.coef_w;
-    // sum over the digit's primes of [x_i (Qd/q_i)^-1]_{q_i} (Qd/q_i mod t), as in modup_body
+    // sum over the digit's primes of v_i (Qd/q_i mod t), v_i = [x_i (Qd/q_i)^-1]_{q_i} from the inverse
+    // transform's store (every target would repeat that product), left below 4t for the butterflies
+    const uint64_t *v = coef + (int64_t)lo * N;
     ntt2_fwd_cols<LOGN>(
-        sm,
-        [&](int64_t x) {
-            uint64_t a = 0;
-            for (int i = 0; i < hi - lo; ++i) {
-                const uint64_t qi = mc[lo + i].q;
-                const uint64_t term = mul_shoup(mul_shoup(coef[(int64_t)(lo + i) * N + x], mu.inv[d][i], mu.inv_shoup[d][i], qi), mu.hat[d][i][u],
-                                                mu.hat_shoup[d][i][u], t);
-                a = i == 0 ? term : add_mod(a, term, t);
-            }
-            return a;
-        },
+        sm, [&](int64_t x) { return conv_lazy(hi - lo, [&](int i) { return v[(int64_t)i * N + x]; }, &mu.hat[d][0][u], &mu.hat_shoup[d][0][u], HE_MAX_LIMBS, t); },
         dst, c0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, t);
 }
 
@@ -1857,7 +1849,7 @@ void launch_rotate_many(he_ctx *ctx, const RotJob *jobs, int count, int level, u
         auto go = [&](auto L, auto NB) {
             constexpr int LG = decltype(L)::value, NB1 = decltype(NB)::value;
             launch_k(rot2_intt_rows_kernel<LG, LG - 6 - NB1>, (unsigned)(count * rg.nl * tiles_r), NTT2_THREADS, 0, st, tab, rg, tw, mc);
-            launch_k(rot2_intt_cols_kernel<LG>, (unsigned)(count * rg.nl * tiles_c), NTT2_THREADS, 0, st, rg, tw, mc);
+            launch_k(rot2_intt_cols_kernel<LG>, (unsigned)(count * rg.nl * tiles_c), NTT2_THREADS, 0, st, rg, mu, tw, mc);
             launch_k(rot2_modup_cols_kernel<LG>, (unsigned)(items * tiles_c), NTT2_THREADS, 0, st, tab, rg, mu, tw, mc);
             launch_k(rot2_modup_rows_kernel<LG>, (unsigned)(items * tiles_r), NTT2_THREADS, 0, st, rg, mu, tw, mc);
         };
