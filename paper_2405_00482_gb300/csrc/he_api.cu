@@ -1174,6 +1174,10 @@ int he_matmult_plain_cipher(he_ctx *ctx, const he_plan *plan, const he_ptmat *pm
         }
     }
     for (int r = 0; r < n_out; ++r) {
+        outs[r].level = level - 1;
+        outs[r].scale = ins[0].scale * pm->scale / (double)ctx->primes[level];
+        // one diagonal, one column block: the product and its rescale in one launch
+        if (!rot && C == 1 && launch_product_rescale(ctx, ins[0].data, pm->data + (size_t)r * pm->ext * N, level, outs[r].data)) continue;
         for (size_t c = 0; c < C; ++c)
             launch_matmult_loop(ctx, pm, r, (int)c, ins[c].data, rot ? D + c * mu.ndig * ext * N : nullptr, acc, cacc, c > 0);
         const uint64_t *pre = cacc;
@@ -1186,8 +1190,6 @@ int he_matmult_plain_cipher(he_ctx *ctx, const he_plan *plan, const he_ptmat *pm
             }
             launch_rescale(ctx, pre, level, outs[r].data, tmp);
         }
-        outs[r].level = level - 1;
-        outs[r].scale = ins[0].scale * pm->scale / (double)ctx->primes[level];
     }
     return last_launch();
 }

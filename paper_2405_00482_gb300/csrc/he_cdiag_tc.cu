@@ -273,11 +273,10 @@ __device__ __forceinline__ void tc_residues(const TcGeom &g, const TcTile &t, in
     }
 }
 __global__ void __launch_bounds__(TC_RES_THREADS, 2) cdiag_tc_residues_kernel(const __grid_constant__ TcGeom g, const TcLimb *__restrict__ limbs, unsigned char *X) {
-    HE_GRID_LAUNCH();
+    HE_GRID_DEP();
     __shared__ const uint64_t *ct[TC_DIAGS];
     for (int i = threadIdx.x; i < g.cnt; i += TC_RES_THREADS) ct[i] = g.ct[i];
     __syncthreads();
-    HE_GRID_WAIT();
     const TcTile t = tc_tile_of(g, g.first + blockIdx.x);
     const TcLimb &lb = limbs[t.u];
     unsigned char *out = X + blockIdx.x * g.tile_bytes;

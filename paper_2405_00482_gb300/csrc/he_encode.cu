@@ -951,9 +951,17 @@ static bool launch_encode_pairs(he_ctx *ctx, SRC src, int count, double scale, i
 }
 
 bool launch_encode_matrix(he_ctx *ctx, const he_plan &p, const double *X, int trans, int count, double scale, int64_t *coeffs) {
-    if (count < 2) return false;
     auto lg = [](int64_t v) { return __builtin_ctzll((unsigned long long)v); };
     const MatrixSrc src{p, X, trans, lg(p.m_prime), lg(p.col_blocks), lg(p.nb), lg(p.mb)};
+    if (count < 2) {  // one diagonal: the single-plaintext form, its slots read from X as well
+        if (count < 1 || fft_cluster_log(ctx->log_n, count) != 3) return false;
+        const float4 *tw = reinterpret_cast<const float4 *>(ctx->d_fft);
+        const float4 *twist = tw + ctx->n / 4;
+        launch_fft_cl<3, 1>(by_logn(ctx->log_n, [](auto L) { return encode_cl_kernel<3, 1, L.value, MatrixSrc>; }), ctx, count, src, scale, tw, twist,
+                            reinterpret_cast<const int32_t *>(twist + ctx->n / 2), coeffs, ctx->log_n);
+        ctx->launches++;
+        return true;
+    }
     if (!launch_encode_pairs(ctx, src, count, scale, coeffs)) return false;
     ctx->launches++;
     return true;
@@ -1143,6 +1151,7 @@ void encode_set_smem_limits(int max_bytes) {
         cudaFuncSetAttribute(decode_cl_kernel<2, 1, L.value, DecodeSlots>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
         cudaFuncSetAttribute(decode_cl_kernel<2, 1, L.value, DecodeRas>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
         cudaFuncSetAttribute(encode_cl_kernel<3, 1, L.value, SlotsSrc>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
+        cudaFuncSetAttribute(encode_cl_kernel<3, 1, L.value, MatrixSrc>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
         cudaFuncSetAttribute(encode_cl_kernel<3, 1, L.value, VectorSrc>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
         cudaFuncSetAttribute(encode_pair_cl_kernel<1, 1, L.value, SlotsSrc>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
         cudaFuncSetAttribute(encode_pair_cl_kernel<2, 1, L.value, SlotsSrc>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);

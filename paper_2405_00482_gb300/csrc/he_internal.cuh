@@ -454,6 +454,9 @@ void launch_moddown(he_ctx *ctx, const uint64_t *x, int level, int ncomp, const 
                     uint64_t *tmp);
 void launch_automorph(he_ctx *ctx, const uint64_t *in, uint64_t *out, int groups, const LimbMap &map, uint32_t g);
 void launch_rescale(he_ctx *ctx, const uint64_t *ct, int level, uint64_t *out, uint64_t *tmp);
+// Rescale(ct (x) pt) in one launch, pt in Montgomery form; false (nothing launched) where that form
+// does not apply
+bool launch_product_rescale(he_ctx *ctx, const uint64_t *ct, const uint64_t *pt, int level, uint64_t *out);
 // ModDown of [2][level+1+K][N] plus add0/add1 (NTT, [level+1][N] each, may be null), then
 // rescale, into out [2][level][N]: one cluster launch when moddown_rescale_fused says so
 bool moddown_rescale_fused(const he_ctx *ctx, int level);

@@ -343,37 +343,69 @@ __global__ void moddown_cl_fused_kernel(const uint64_t *__restrict__ x, int ext,
     }
 }
 
-// rescale of component c, output limb j < level: the last limb in coefficient form (here),
-// centred, reduced mod q_j, NTT, out = (c_j - v) q_l^-1
+// rescale of component c, output limb j < level: the last limb to coefficient form, centred, reduced
+// mod q_j, NTT, out = (c_j - v) q_l^-1.  The inverse transform's cross-CTA stages, the map to q_j and
+// the forward transform's cross-CTA stages are one pass (ntt_cross_inv_fwd), as in ModUp with one limb
+// per digit.  With PT the input is the product ct (x) pt (pt in Montgomery form, [>= level+1][N]),
+// formed as it is loaded: a MatMult of one diagonal in one launch (N = 2^12, two limbs: 6.9 us a call,
+// 12.7 with the loop kernel and a rescale of two passes before it).  ct and pt are written by earlier
+// launches and must not be read before the wait: no __restrict__ on them, which would let their loads
+// be taken for invariant and moved above it.
 // LOGN > 0: the ring size at compile time (logn_rt == LOGN)
-template <int LOGN = 0>
-__global__ void rescale_cl_fused_kernel(const uint64_t *__restrict__ ct, int level, RescaleConst rc, uint64_t *out,
-                                        const uint64_t *__restrict__ d_tw, const ModConst *__restrict__ mc, int logn_rt) {
-    HE_GRID_DEP();
+template <int LOGN, bool PT>
+__global__ void rescale_cl_fused_kernel(const uint64_t *ct, const uint64_t *pt, int level,
+                                        const __grid_constant__ RescaleConst rc, uint64_t *out, const uint64_t *__restrict__ d_tw,
+                                        const ModConst *__restrict__ mc, int logn_rt) {
+    HE_GRID_LAUNCH();
     const int logn = LOGN ? LOGN : logn_rt;
     extern __shared__ uint64_t s[];
     const int N = 1 << logn;
     int item, off, len;
     slice_of<true>(logn, item, off, len);
     const int c = item / level, j = item % level;
-    const uint64_t q = mc[j].q, ql = mc[level].q;
-    uint64_t *lc = cl_acc_slice(s, logn);
-    cl_intt_slice<LOGN>(s, ct + ((int64_t)c * (level + 1) + level) * N + off, level, d_tw, mc, logn, len);
-    for (int k = threadIdx.x; k < len; k += blockDim.x) lc[k] = mul_shoup(s[SIDX(k)], mc[level].ninv, mc[level].ninv_shoup, ql);
-    __syncthreads();
-    const ulonglong2 *tw = twiddles(d_tw, j, 0, logn);
-    tw_prefetch<true, true>(s, tw, logn);
-    for (int k = threadIdx.x; k < len; k += blockDim.x) {
-        uint64_t r = lc[k] + rc.half;
-        if (r >= rc.ql) r -= rc.ql;
-        const int64_t centred = (int64_t)r - (int64_t)rc.half;
-        s[SIDX(k)] = reduce_signed(centred, q, mc[j].mu);
+    const uint64_t q = mc[j].q, ql = mc[level].q, qinv = mc[j].qinv, mu = mc[j].mu;
+    const ulonglong2 *itw = twiddles(d_tw, level, 1, logn), *tw = twiddles(d_tw, j, 0, logn);
+    tw_prefetch<true, false>(s, itw, logn);  // context tables, before the wait
+    ulonglong2 wi[3], wf[3];
+    cross_tw_load<false>(wi, itw);
+    cross_tw_load<true>(wf, tw);
+    HE_GRID_WAIT();
+    const uint64_t *cl = ct + ((int64_t)c * (level + 1) + level) * N + off, *pl = PT ? pt + (int64_t)level * N + off : nullptr;
+    const uint64_t *cj = ct + ((int64_t)c * (level + 1) + j) * N + off, *pj = PT ? pt + (int64_t)j * N + off : nullptr;
+    // the combination's inputs of the first two iterations, in flight during the transforms
+    uint64_t xv[2], pv[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int k = threadIdx.x + r * blockDim.x;
+        if (k < len) {
+            xv[r] = cj[k];
+            pv[r] = PT ? pj[k] : 0;
+        }
     }
+    for (int k = threadIdx.x; k < len; k += blockDim.x) s[SIDX(k)] = PT ? mont_mul(cl[k], pl[k], ql, mc[level].qinv) : cl[k];
     __syncthreads();
-    ntt_fwd_cluster<LOGN>(s, tw, q, logn);
-    const uint64_t *cj = ct + ((int64_t)c * (level + 1) + j) * N + off;
+    ntt_inv_cluster_local<LOGN>(s, ql, logn);
+    tw_prefetch<true, true>(s, tw, logn);  // the inverse copy is no longer read
+    cg::this_cluster().sync();
+    const uint64_t ni = mc[level].ninv, nis = mc[level].ninv_shoup;
+    ntt_cross_inv_fwd(
+        s, wi, ql,
+        [&](uint64_t x) {
+            uint64_t r = mul_shoup(x, ni, nis, ql) + rc.half;
+            if (r >= rc.ql) r -= rc.ql;
+            return reduce_signed((int64_t)r - (int64_t)rc.half, q, mu);
+        },
+        wf, q, logn);
+    tw_slice_wait();
+    cg::this_cluster().sync();
+    ntt_fwd_cluster_local<LOGN>(s, q, logn);
     uint64_t *o = out + ((int64_t)c * level + j) * N + off;
-    for (int k = threadIdx.x; k < len; k += blockDim.x) o[k] = mul_shoup(sub_mod(cj[k], s[SIDX(k)], q), rc.inv[j], rc.inv_shoup[j], q);
+    int r = 0;
+    for (int k = threadIdx.x; k < len; k += blockDim.x, ++r) {
+        uint64_t x = r == 0 ? xv[0] : (r == 1 ? xv[1] : cj[k]);
+        if (PT) x = mont_mul(x, r == 0 ? pv[0] : (r == 1 ? pv[1] : pj[k]), q, qinv);
+        o[k] = mul_shoup(sub_mod(x, s[SIDX(k)], q), rc.inv[j], rc.inv_shoup[j], q);
+    }
 }
 
 // ModDown then rescale (the MatMult epilogue).  Component c, output limb j < L (L = md.nq - 1,
@@ -1608,8 +1640,9 @@ void launch_rescale(he_ctx *ctx, const uint64_t *ct, int level, uint64_t *out, u
     const RescaleConst rc = make_rescale_const(ctx, level);
     ctx->launches++;
     if (use_cluster(ctx->log_n, 2 * level)) {  // the inverse NTT of the last limb happens inside
-        launch_cluster(by_logn(ctx->log_n, [](auto L) { return rescale_cl_fused_kernel<L.value>; }), 2 * level * HE_NTT_CL_SIZE, cl_threads(ctx->log_n), cl_fused_smem_bytes(ctx->log_n), ctx->stream,
-                       ct, level, rc, out, (const uint64_t *)ctx->d_tw, (const ModConst *)ctx->d_mc, ctx->log_n);
+        launch_cluster(by_logn(ctx->log_n, [](auto L) { return rescale_cl_fused_kernel<L.value, false>; }), 2 * level * HE_NTT_CL_SIZE,
+                       cl_threads(ctx->log_n), cl_smem_bytes(ctx->log_n), ctx->stream, ct, (const uint64_t *)nullptr, level, rc, out,
+                       (const uint64_t *)ctx->d_tw, (const ModConst *)ctx->d_mc, ctx->log_n);
         return;
     }
     LimbMap lmap{};
@@ -1619,6 +1652,15 @@ void launch_rescale(he_ctx *ctx, const uint64_t *ct, int level, uint64_t *out, u
     launch_ntt_inv_strided(ctx, ct + (int64_t)level * N, (int64_t)(level + 1) * N, tmp, N, 2, lmap);
     launch_k(rescale_kernel<false>, 2 * level, ntt_threads(ctx->log_n), ntt_smem_bytes(ctx->log_n), ctx->stream, ct, level, tmp, rc, out, ctx->d_tw,
              ctx->d_mc, ctx->log_n);
+}
+
+bool launch_product_rescale(he_ctx *ctx, const uint64_t *ct, const uint64_t *pt, int level, uint64_t *out) {
+    if (!use_cluster(ctx->log_n, 2 * level)) return false;
+    ctx->launches++;
+    launch_cluster(by_logn(ctx->log_n, [](auto L) { return rescale_cl_fused_kernel<L.value, true>; }), 2 * level * HE_NTT_CL_SIZE, cl_threads(ctx->log_n),
+                   cl_smem_bytes(ctx->log_n), ctx->stream, ct, pt, level, make_rescale_const(ctx, level), out, (const uint64_t *)ctx->d_tw,
+                   (const ModConst *)ctx->d_mc, ctx->log_n);
+    return true;
 }
 
 bool moddown_rescale_fused(const he_ctx *ctx, int level) { return level >= 1 && use_cluster(ctx->log_n, 2 * level); }
@@ -1891,7 +1933,10 @@ void ops_set_smem_limits(int max_bytes) {
         cudaFuncSetAttribute(batch_mdr_ntt_cl_kernel<L.value>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
     });
     each_logn([max_bytes](auto L) { cudaFuncSetAttribute(moddown_cl_fused_kernel<L.value>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes); });
-    each_logn([max_bytes](auto L) { cudaFuncSetAttribute(rescale_cl_fused_kernel<L.value>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes); });
+    each_logn([max_bytes](auto L) {
+        cudaFuncSetAttribute(rescale_cl_fused_kernel<L.value, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
+        cudaFuncSetAttribute(rescale_cl_fused_kernel<L.value, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
+    });
     each_logn([max_bytes](auto L) { cudaFuncSetAttribute(moddown_rescale_intt_kernel<L.value>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes); });
     each_logn([max_bytes](auto L) { cudaFuncSetAttribute(moddown_rescale_ntt_kernel<L.value>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes); });
 
