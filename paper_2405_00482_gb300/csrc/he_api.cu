@@ -126,6 +126,9 @@ ModConst make_modconst(uint64_t q, int log_n) {
     m.p40_shoup = shoup(m.p40, q);
     m.p80 = hpow(2, 80, q);
     m.p80_shoup = shoup(m.p80, q);
+    const uint64_t two60 = (uint64_t)1 << 60, two40 = (uint64_t)1 << 40;
+    m.lift = q >> 58 ? 4 * q : (two60 + q - 1) / q * q;
+    m.delta40 = q < two40 && two40 - q < (1u << 23) ? two40 - q : 0;
     return m;
 }
 

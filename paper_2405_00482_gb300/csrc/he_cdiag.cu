@@ -167,14 +167,14 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) cdiag_rescale_cols_kernel(con
     __shared__ uint64_t sm[ntt2_cols_smem_words()];
     const int item = blockIdx.x / TILES, c0 = (blockIdx.x % TILES) * NTT2_TC;
     const int kl = item / (2 * level), c = (item / level) % 2, j = item % level;
-    const uint64_t q = mc[j].q, mu = mc[j].mu, half = ql / 2;
+    const uint64_t q = mc[j].q, mu = mc[j].mu, lift = mc[j].lift, half = ql / 2;
     const uint64_t *lc = last + ((int64_t)(k_first + kl) * 2 + c) * N;
     ntt2_fwd_cols<LOGN>(
-        sm,
-        [=](int64_t x) {
-            uint64_t r = lc[x] + half;
+        sm, [=](int64_t x) { return lc[x]; },
+        [=](uint64_t v) {
+            uint64_t r = v + half;
             if (r >= ql) r -= ql;
-            return reduce_signed((int64_t)r - (int64_t)half, q, mu);
+            return lift_signed((int64_t)r - (int64_t)half, q, lift, mu);
         },
         outs.p[kl] + ((int64_t)c * level + j) * N, c0, TwGlobal{twiddles(d_tw, j, 0, LOGN)}, q);
 }
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) cdiag_rescale_rows_kernel(con
     const uint64_t q = mc[j].q, inv = rc.inv[j], invs = rc.inv_shoup[j];
     const uint64_t *cj = pre + (((int64_t)(k_first + kl) * 2 + c) * (level + 1) + j) * N;
     uint64_t *o = outs.p[kl] + ((int64_t)c * level + j) * N;
-    ntt2_fwd_rows<LOGN>(sm, o, b0, TwGlobal{twiddles(d_tw, j, 0, LOGN)}, q, mc[j].mu,
+    ntt2_fwd_rows<LOGN>(sm, o, b0, TwGlobal{twiddles(d_tw, j, 0, LOGN)}, mc[j],
                         [=](int x, uint64_t v) { o[x] = mul_shoup(sub_mod(cj[x], v, q), inv, invs, q); });
 }
 

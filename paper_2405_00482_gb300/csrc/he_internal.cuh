@@ -90,6 +90,24 @@ __device__ __forceinline__ uint64_t reduce_signed(int64_t v, uint64_t q, uint64_
     return q - 1 - r;
 }
 
+// a signed v as a transform's input (congruent, not reduced): at most 4q for q >= 2^58, below 2^61 for
+// smaller primes, whose butterflies skip the correction (ntt_fwd_radix).  Values past 2^60 in
+// magnitude, which no encoding in use reaches, are reduced.
+__device__ __forceinline__ uint64_t lift_signed(int64_t v, uint64_t q, uint64_t lift, uint64_t mu) {
+    if ((uint64_t)v + (1ull << 60) > (1ull << 61)) return reduce_signed(v, q, mu);
+    return (uint64_t)v + (v < 0 ? lift : 0);
+}
+// x mod q for q = 2^40 - delta, delta < 2^23: 2^40 = delta folds any 64-bit x below 2^47, then below
+// q + 2^31 (half the instructions of a Barrett step)
+__device__ __forceinline__ uint64_t reduce40(uint64_t x, uint64_t q, uint32_t delta) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const uint32_t hi = (uint32_t)(x >> 32);
+        x = (uint64_t)(hi >> 8) * delta + (((uint64_t)(hi & 0xFF) << 32) | (uint32_t)x);
+    }
+    return x >= q ? x - q : x;
+}
+
 // position of the NTT-domain slot k after the automorphism X -> X^g (bit-reversed order):
 // out[k] = in[automorph_src(k, g)], exponent e_k = 2 brv(k) + 1.
 __device__ __forceinline__ uint32_t automorph_src(uint32_t k, uint32_t g, int logn) {
@@ -109,6 +127,8 @@ struct ModConst {
     uint64_t mu;      // floor(2^64 / q), for reduce_barrett
     uint64_t r1, r1_shoup;  // 2^64 mod q with its Shoup quotient: x -> x 2^64 mod q (Montgomery form)
     uint64_t p40, p40_shoup, p80, p80_shoup;  // 2^40 and 2^80 mod q: recombination of byte-split products (he_bconv.cu)
+    uint64_t lift;     // a multiple of q: 4q from 2^58, else the first from 2^60 (lift_signed)
+    uint64_t delta40;  // 2^40 - q when 0 < 2^40 - q < 2^23 (reduce40), else 0
 };
 
 // next start/end event pair of profiled kernel class `kind` (HE_PROF_*), or nullptr when profiling is off

@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) ks2_conv_cols_kernel(KsGeom k
             for (int i = 1; i < kg.K; ++i) v = add_mod(v, mul_shoup(pc[(int64_t)i * N + x], md.hat[i][l], md.hat_shoup[i][l], q), q);
             return v;
         },
-        cv + (int64_t)item * N, c0, TwGlobal{twiddles(d_tw, pl, 0, LOGN)}, q);
+        [](uint64_t v) { return v; }, cv + (int64_t)item * N, c0, TwGlobal{twiddles(d_tw, pl, 0, LOGN)}, q);
 }
 
 template <int LOGN>
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) ks2_conv_rows_kernel(uint64_t
     __shared__ uint64_t sm[ntt2_frows_smem_words(LOGN - 6)];
     const int item = blockIdx.x / TILES, b0 = (blockIdx.x % TILES) * NTT2_TR;
     const int pl = md.q_prime[item % nl];
-    ntt2_fwd_rows<LOGN>(sm, cv + (int64_t)item * N, b0, TwGlobal{twiddles(d_tw, pl, 0, LOGN)}, mc[pl].q, mc[pl].mu);
+    ntt2_fwd_rows<LOGN>(sm, cv + (int64_t)item * N, b0, TwGlobal{twiddles(d_tw, pl, 0, LOGN)}, mc[pl]);
 }
 
 // the four launches of transform variant 2 (log N = 12, 13, 14)

@@ -166,15 +166,23 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) ntt2_cols_kernel(const void *
     __shared__ uint64_t sm[ntt2_cols_smem_words()];
     const int poly = blockIdx.x / TILES, c0 = (blockIdx.x % TILES) * NTT2_TC;
     const int g = poly / map.n, l = poly % map.n, p = map.prime[l];
-    const uint64_t q = mc[p].q, r1 = mc[p].r1, r1s = mc[p].r1_shoup, mu = mc[p].mu;
+    // x 2^64 mod q (to_mont) by an unreduced product on the input: as the product that ends the row
+    // phase it cost 1 us of 36 more (256 limb-polys of N = 2^13), that phase being the longer one
+    const uint64_t q = mc[p].q, lift = mc[p].lift, mu = mc[p].mu, r1 = mc[p].r1, r1s = mc[p].r1_shoup;
     uint64_t *dst = out + g * out_gs + (int64_t)l * N;
     if constexpr (I64) {  // int64 coefficients, shared by the limbs of group g, reduced mod q
         const int64_t *src = static_cast<const int64_t *>(in_v) + g * in_gs;
-        ntt2_fwd_cols<LOGN>(sm, [=](int64_t x) { return to_mont ? signed_to_mont(src[x], r1, r1s, q) : reduce_signed(src[x], q, mu); }, dst, c0,
+        ntt2_fwd_cols<LOGN>(sm, 
+            [=](int64_t x) { return src[x]; },
+            [=](uint64_t w) {
+                const uint64_t v = lift_signed((int64_t)w, q, lift, mu);
+                return to_mont ? mul_shoup_lazy(v, r1, r1s, q) : v;
+            },
+            dst, c0,
                             TwGlobal{twiddles(d_tw, p, 0, LOGN)}, q);
     } else {
         const uint64_t *src = static_cast<const uint64_t *>(in_v) + g * in_gs + (int64_t)l * N;
-        ntt2_fwd_cols<LOGN>(sm, [=](int64_t x) { return to_mont ? mul_shoup(src[x], r1, r1s, q) : src[x]; }, dst, c0,
+        ntt2_fwd_cols<LOGN>(sm, [=](int64_t x) { return src[x]; }, [=](uint64_t v) { return to_mont ? mul_shoup_lazy(v, r1, r1s, q) : v; }, dst, c0,
                             TwGlobal{twiddles(d_tw, p, 0, LOGN)}, q);
     }
 }
@@ -188,9 +196,9 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) ntt2_cols_tab_kernel(const in
     __shared__ uint64_t sm[ntt2_cols_smem_words()];
     const int poly = blockIdx.x / TILES, c0 = (blockIdx.x % TILES) * NTT2_TC;
     const int g = poly / map.n, l = poly % map.n, p = map.prime[l];
-    const uint64_t q = mc[p].q, mu = mc[p].mu;
+    const uint64_t q = mc[p].q, lift = mc[p].lift, mu = mc[p].mu;
     const int64_t *src = in + (int64_t)g * N;
-    ntt2_fwd_cols<LOGN>(sm, [=](int64_t x) { return reduce_signed(src[x], q, mu); }, outs.p[g] + (int64_t)l * N, c0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, q);
+    ntt2_fwd_cols<LOGN>(sm, [=](int64_t x) { return src[x]; }, [=](uint64_t v) { return lift_signed((int64_t)v, q, lift, mu); }, outs.p[g] + (int64_t)l * N, c0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, q);
 }
 template <int LOGN>
 __global__ void __launch_bounds__(NTT2_THREADS, 8) ntt2_rows_tab_kernel(const __grid_constant__ OutPtrs outs, LimbMap map, const uint64_t *__restrict__ d_tw,
@@ -200,7 +208,7 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) ntt2_rows_tab_kernel(const __
     __shared__ uint64_t sm[ntt2_frows_smem_words(LOGN - 6)];
     const int poly = blockIdx.x / TILES, b0 = (blockIdx.x % TILES) * NTT2_TR;
     const int g = poly / map.n, l = poly % map.n, p = map.prime[l];
-    ntt2_fwd_rows<LOGN>(sm, outs.p[g] + (int64_t)l * N, b0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, mc[p].q, mc[p].mu);
+    ntt2_fwd_rows<LOGN>(sm, outs.p[g] + (int64_t)l * N, b0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, mc[p]);
 }
 
 template <int LOGN>
@@ -211,7 +219,7 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) ntt2_rows_kernel(uint64_t *da
     __shared__ uint64_t sm[ntt2_frows_smem_words(LOGN - 6)];
     const int poly = blockIdx.x / TILES, b0 = (blockIdx.x % TILES) * NTT2_TR;
     const int g = poly / map.n, l = poly % map.n, p = map.prime[l];
-    ntt2_fwd_rows<LOGN>(sm, data + g * gs + (int64_t)l * N, b0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, mc[p].q, mc[p].mu);
+    ntt2_fwd_rows<LOGN>(sm, data + g * gs + (int64_t)l * N, b0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, mc[p]);
 }
 
 // inverse: rows (in to out), then columns in place with the factor N^-1

@@ -97,8 +97,9 @@ struct TwFirstInv {
 // at stage s0 + j element k meets twiddle entry m + (g << j) + (k >> (NB - j)), m = 2^(s0+j),
 // the 2^j consecutive entries loaded once per stage.  Harvey's lazy butterfly: inputs below 4q,
 // outputs below 4q.  Without CORR the top input is not brought below 2q first: each stage then
-// adds less than 2q to the bound, so inputs below 4q stay below (4 + 2 log N) q, which fits in
-// 64 bits for q < 2^59 and log N <= 14 (the caller reduces at the end).
+// adds less than 2q to the bound, so for log N <= 14 inputs below 4q stay below 32 q, which fits in
+// 64 bits for q < 2^59, and inputs below 2^61 below 2^61 + 28 q, which fits for q < 2^58 (the caller
+// reduces at the end).
 template <int NB, class TWA, bool CORR = true>
 __device__ __forceinline__ void ntt_fwd_radix(uint64_t (&r)[1 << NB], TWA tw, uint64_t q, int s0, int g) {
     constexpr int E = 1 << NB;
@@ -377,17 +378,10 @@ __host__ __device__ constexpr int ntt2_rows_smem_words(int lb) { return NTT2_TR 
 __host__ __device__ constexpr int ntt2_frows_smem_words(int lb) { return NTT2_TR * (1 << lb) + NTT2_TR * (1 << lb) / 32; }
 __device__ __forceinline__ int ntt2_at(int m) { return m + (m >> 3); }
 
-// canonical residue of v 2^64 mod q for a signed v (Shoup product by 2^64 mod q of |v|)
-__device__ __forceinline__ uint64_t signed_to_mont(int64_t v, uint64_t r1, uint64_t r1s, uint64_t q) {
-    const uint64_t a = v >= 0 ? (uint64_t)v : 0ull - (uint64_t)v;
-    const uint64_t r = mul_shoup(a, r1, r1s, q);
-    return (v < 0 && r != 0) ? q - r : r;
-}
-
-// forward stages 0-5 of columns c0 .. c0 + NTT2_TC - 1 of one limb-poly: load(x) gives the
-// input of element x, below 4q; writes the stage-5 values to dst[x]
-template <int LOGN, class LOAD>
-__device__ __forceinline__ void ntt2_fwd_cols(uint64_t *sm, LOAD load, uint64_t *dst, int c0, TwGlobal tw, uint64_t q) {
+// forward stages 0-5 of columns c0 .. c0 + NTT2_TC - 1 of one limb-poly, inputs below 4q (or lift_signed's),; writes the stage-5 values to dst[x]
+// input of element x from the word at x: prep(load(x)), all eight loads of a thread before the first prep
+template <int LOGN, class LOAD, class PREP>
+__device__ __forceinline__ void ntt2_fwd_cols(uint64_t *sm, LOAD load, PREP prep, uint64_t *dst, int c0, TwGlobal tw, uint64_t q) {
     constexpr int C = (1 << LOGN) >> 6, PAD = NTT2_TC + 1;
     static_assert(NTT2_THREADS == 8 * NTT2_TC, "one thread per (column, set of 8)");
     const int c = threadIdx.x % NTT2_TC, r = threadIdx.x / NTT2_TC;
@@ -395,7 +389,9 @@ __device__ __forceinline__ void ntt2_fwd_cols(uint64_t *sm, LOAD load, uint64_t 
     uint64_t v[8];
     // stages 0-2 on the column's elements l = r + 8 i (one group at stage 0)
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = load((int64_t)(r + 8 * i) * C + c0 + c);
+    for (int i = 0; i < 8; ++i) v[i] = (uint64_t)load((int64_t)(r + 8 * i) * C + c0 + c);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = prep(v[i]);
     if (corr) ntt_fwd_radix<3, TwGlobal, true>(v, tw, q, 0, 0);
     else ntt_fwd_radix<3, TwGlobal, false>(v, tw, q, 0, 0);
 #pragma unroll
@@ -415,9 +411,10 @@ __device__ __forceinline__ void ntt2_fwd_cols(uint64_t *sm, LOAD load, uint64_t 
 // slice [b0 R, (b0 + NTT2_TR) R) of the transform and run through the one-CTA form's passes of up
 // to three stages (ntt_fwd_pass over the sets whose elements fall in the slice, as a cluster
 // member does), so a thread holds 8 values at a time.  Element x's canonical result v goes to
-// store(x, v) (the form without it writes it back in place).
+// store(x, v) (the short form writes it back in place).
 template <int LOGN, class STORE>
-__device__ __forceinline__ void ntt2_fwd_rows(uint64_t *sm, const uint64_t *poly, int b0, TwGlobal tw, uint64_t q, uint64_t mu, STORE store) {
+__device__ __forceinline__ void ntt2_fwd_rows(uint64_t *sm, const uint64_t *poly, int b0, TwGlobal tw, const ModConst &m, STORE store) {
+    const uint64_t q = m.q;
     constexpr int LB = LOGN - 6, R = 1 << LB, LEN = NTT2_TR * R;
     const int off = b0 * R;  // a multiple of 32, so SIDX splits over the offset
     stage_in(sm, poly + off, LEN, [](uint64_t v) { return v; });
@@ -446,15 +443,23 @@ __device__ __forceinline__ void ntt2_fwd_rows(uint64_t *sm, const uint64_t *poly
             else ntt_fwd_pass<1, TwGlobal, false>(sm, tw, q, LOGN, s0, false, off >> 1, (off + LEN) >> 1, off);
         }
     }
-    // without the lazy correction the values are below (4 + 2 log N) q: one Barrett step
-    for (int k = threadIdx.x; k < LEN; k += NTT2_THREADS) {
-        const uint64_t v = sm[SIDX(k)];
-        store(off + k, corr ? v : reduce_barrett(v, q, mu));
+    // with the lazy correction the last pass left canonical values; without, they are below 2^64
+    const uint64_t mu = m.mu;
+    const uint32_t delta = (uint32_t)m.delta40;
+    if (corr) {
+#pragma unroll 4
+        for (int k = threadIdx.x; k < LEN; k += NTT2_THREADS) store(off + k, sm[SIDX(k)]);
+    } else if (delta) {
+#pragma unroll 4
+        for (int k = threadIdx.x; k < LEN; k += NTT2_THREADS) store(off + k, reduce40(sm[SIDX(k)], q, delta));
+    } else {
+#pragma unroll 4
+        for (int k = threadIdx.x; k < LEN; k += NTT2_THREADS) store(off + k, reduce_barrett(sm[SIDX(k)], q, mu));
     }
 }
 template <int LOGN>
-__device__ __forceinline__ void ntt2_fwd_rows(uint64_t *sm, uint64_t *poly, int b0, TwGlobal tw, uint64_t q, uint64_t mu) {
-    ntt2_fwd_rows<LOGN>(sm, poly, b0, tw, q, mu, [=](int x, uint64_t v) { poly[x] = v; });
+__device__ __forceinline__ void ntt2_fwd_rows(uint64_t *sm, uint64_t *poly, int b0, TwGlobal tw, const ModConst &m) {
+    ntt2_fwd_rows<LOGN>(sm, poly, b0, tw, m, [=](int x, uint64_t v) { poly[x] = v; });
 }
 
 // inverse stages 0 .. log N - 7 of rows b0 .. b0 + NTT2_TR - 1 of one limb-poly (inputs below 2q),

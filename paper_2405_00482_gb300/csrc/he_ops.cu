@@ -628,7 +628,7 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) rot2_modup_cols_kernel(const 
     const uint64_t *v = coef + (int64_t)lo * N;
     ntt2_fwd_cols<LOGN>(
         sm, [&](int64_t x) { return conv_lazy(hi - lo, [&](int i) { return v[(int64_t)i * N + x]; }, &mu.hat[d][0][u], &mu.hat_shoup[d][0][u], HE_MAX_LIMBS, t); },
-        dst, c0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, t);
+        [](uint64_t w) { return w; }, dst, c0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, t);
 }
 
 template <int LOGN>
@@ -642,7 +642,7 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) rot2_modup_rows_kernel(RotGeo
     const int lo = d * mu.alpha, hi = lo + mu.alpha < mu.nq ? lo + mu.alpha : mu.nq;
     if (u >= lo && u < hi) return;  // copied, already in NTT form
     const int p = mu.ext_prime[u];
-    ntt2_fwd_rows<LOGN>(sm, rg.D + j * rg.d_w + ((int64_t)d * mu.ext + u) * N, b0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, mc[p].q, mc[p].mu);
+    ntt2_fwd_rows<LOGN>(sm, rg.D + j * rg.d_w + ((int64_t)d * mu.ext + u) * N, b0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, mc[p]);
 }
 
 // ModUp of the jobs' c1 (NTT form) as clusters, item (j, d, u), the inverse NTT inside: for
