@@ -731,7 +731,7 @@ int he_rotate_hoisted(he_ctx *ctx, const he_ct *in, const int32_t *steps, int k,
             return HE_ECUDA;
     const int n_jobs = (int)jobs.size();
     if (n_jobs > 0) {
-        // one ModUp of c1 (O4), then the key switch of every rotation, two launches per 64
+        // one ModUp of c1 (O4), then the key switch of every rotation, two launches per 128
         const ModUpConst &mu = ctx->modup[level];
         const size_t wD = (size_t)mu.ndig * mu.ext * N, wc = nl * N, wp = keyswitch_many_pc_words(ctx, n_jobs);
         uint64_t *s = ctx_scratch(ctx, wD + wc + wp);
@@ -1069,7 +1069,8 @@ static int fuse_try(he_ctx *ctx, he_ptmat *pm, const uint64_t *ct, const uint64_
     }
     const int rc = tune_matmult_fused(ctx, pm, ct, D, acc, cacc);
     if (rc != HE_OK) return rc;
-    if (pm->fvariant >= 0 && pm->fuse_ms[pm->fvariant] < pm->tune_ms[pm->variant]) {
+    const float unfused = pm->rows_ms > 0.0f && 0.5f * pm->rows_ms < pm->tune_ms[pm->variant] ? 0.5f * pm->rows_ms : pm->tune_ms[pm->variant];
+    if (pm->fvariant >= 0 && pm->fuse_ms[pm->fvariant] < unfused) {
         pm->fuse_state = 1;
         return HE_OK;
     }
@@ -1153,14 +1154,23 @@ int he_matmult_plain_cipher(he_ctx *ctx, const he_plan *plan, const he_ptmat *pm
     const bool rot = p.m_prime > 1;
     const size_t wD = rot ? C * mu.ndig * ext * N : 0, wc = nl * N, wa = 2 * ext * N, wcc = 2 * nl * N, wsum = 2 * nl * N,
                  wt = 2 * (ctx->K > 1 ? ctx->K : 1) * N + 2 * N;
-    uint64_t *s = ctx_scratch(ctx, wD + wc + wa + wcc + wsum + wt);
+    // row blocks in pairs want a second accumulator: scratch that cannot grow (no memory, a stream
+    // under capture) takes them one by one
+    const size_t need = wD + wc + wa + wcc + wsum + wt;
+    bool pairs = mm_rows_fit(ctx, pm) && (need + wa <= ctx->scratch_words || !capturing(ctx->stream));
+    uint64_t *s = pairs ? ctx_scratch(ctx, need + wa) : nullptr;
+    if (!s) {
+        cudaGetLastError();
+        pairs = false;
+        s = ctx_scratch(ctx, need);
+    }
     if (!s) return HE_ENOMEM;
-    uint64_t *D = s, *coef = D + wD, *acc = coef + wc, *cacc = acc + wa, *sum = cacc + wcc, *tmp = sum + wsum;
+    uint64_t *D = s, *coef = D + wD, *cacc = coef + wc, *sum = cacc + wcc, *tmp = sum + wsum, *acc = tmp + wt;
     if (rot)
         for (size_t c = 0; c < C; ++c) launch_modup(ctx, ins[c].data + nl * N, level, D + c * mu.ndig * ext * N, coef);
     if (pm->variant < 0) {
         if (rot) {
-            rc = tune_matmult_loop(ctx, pm, ins[0].data, D, acc, cacc);
+            rc = tune_matmult_loop(ctx, pm, ins[0].data, D, acc, cacc, pairs);
             if (rc != HE_OK) return rc;
         } else {
             pm->variant = 0;
@@ -1176,23 +1186,37 @@ int he_matmult_plain_cipher(he_ctx *ctx, const he_plan *plan, const he_ptmat *pm
             if (rc != HE_OK) return rc;
         }
     }
+    const bool fk = pm->fuse_state == 1 && pm->fused && pm->fused_gen == pm->enc_gen && pm->fvariant >= 0;
+    pairs = pairs && !fk && pm->rows_ms > 0.0f;
+    // ModDown of x with the unrotated part (may be null) added, and rescale, into outs[r]
+    auto finish = [&](int r, const uint64_t *x, const uint64_t *add) {
+        const uint64_t *add1 = add ? add + nl * N : nullptr;
+        if (moddown_rescale_fused(ctx, level)) {
+            launch_moddown_rescale(ctx, x, level, add, add1, outs[r].data, tmp);
+            return;
+        }
+        launch_moddown(ctx, x, level, 2, add, add1, sum, tmp);
+        launch_rescale(ctx, sum, level, outs[r].data, tmp);
+    };
     for (int r = 0; r < n_out; ++r) {
         outs[r].level = level - 1;
         outs[r].scale = ins[0].scale * pm->scale / (double)ctx->primes[level];
+    }
+    for (int r = 0; r < n_out; ++r) {
+        if (pairs && r + 1 < n_out) {
+            for (size_t c = 0; c < C; ++c) launch_matmult_rows(ctx, pm, r, (int)c, ins[c].data, D + c * mu.ndig * ext * N, acc, c > 0);
+            finish(r, acc, nullptr);
+            finish(++r, acc + wa, nullptr);
+            continue;
+        }
         // one diagonal, one column block: the product and its rescale in one launch
         if (!rot && C == 1 && launch_product_rescale(ctx, ins[0].data, pm->data + (size_t)r * pm->ext * N, level, outs[r].data)) continue;
         for (size_t c = 0; c < C; ++c)
             launch_matmult_loop(ctx, pm, r, (int)c, ins[c].data, rot ? D + c * mu.ndig * ext * N : nullptr, acc, cacc, c > 0);
-        const uint64_t *pre = cacc;
-        if (rot && moddown_rescale_fused(ctx, level)) {
-            launch_moddown_rescale(ctx, acc, level, cacc, cacc + nl * N, outs[r].data, tmp);
-        } else {
-            if (rot) {
-                launch_moddown(ctx, acc, level, 2, cacc, cacc + nl * N, sum, tmp);
-                pre = sum;
-            }
-            launch_rescale(ctx, pre, level, outs[r].data, tmp);
-        }
+        if (rot)
+            finish(r, acc, cacc);
+        else
+            launch_rescale(ctx, cacc, level, outs[r].data, tmp);
     }
     return last_launch();
 }
@@ -1426,6 +1450,7 @@ int he_ptmat_tuning(const he_ptmat *pm, int *variant, float *ms) {
 int he_ptmat_set_variant(he_ptmat *pm, int v) {
     if (!pm || v < -1 || v >= mm_variant_count()) return HE_EINVAL;
     pm->variant = v;
+    pm->rows_ms = 0.0f;  // row blocks one by one, with this variant
     return HE_OK;
 }
 

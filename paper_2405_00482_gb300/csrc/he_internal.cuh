@@ -311,6 +311,7 @@ struct he_ptmat {
     int fvariant = -1;       // staged variant of the fused form chosen by timing
     int fvariant_pin = -1;   // >= 0: fused form with this variant, built without timing
     float fuse_ms[HE_MM_MAX_VARIANTS] = {};
+    float rows_ms = 0.0f;    // > 0: the unfused product takes its row blocks in pairs (milliseconds of a pair)
     uint64_t enc_gen = 0;    // bumped by every (re-)encoding of data
     uint64_t fused_gen = 0;  // enc_gen the fused tables were built from
     uint64_t mm_gen = ~0ull; // enc_gen at the last MatMult
@@ -361,7 +362,7 @@ int mm_variant_count();
 int mm_variant_tile(int v);  // coefficients per tile of loop-kernel variant v
 void mm_variant_shape(int v, int *vec, int *grp, int *stages, int *ga);
 int mm_batch_ctas_per_sm(int v, int ndig);
-int tune_matmult_loop(he_ctx *ctx, he_ptmat *pm, const uint64_t *ct, const uint64_t *D, uint64_t *acc, uint64_t *cacc);
+int tune_matmult_loop(he_ctx *ctx, he_ptmat *pm, const uint64_t *ct, const uint64_t *D, uint64_t *acc, uint64_t *cacc, bool rows);
 int tune_matmult_fused(he_ctx *ctx, he_ptmat *pm, const uint64_t *ct, const uint64_t *D, uint64_t *acc, uint64_t *cacc);
 bool capturing(cudaStream_t st);           // st is being captured into a graph
 bool mm_variant_fusable(int v, int ndig);  // variant v has a fused-key form for ndig digits
@@ -484,6 +485,10 @@ void launch_moddown_rescale(he_ctx *ctx, const uint64_t *x, int level, const uin
                             uint64_t *tmp);  // tmp: 2 (K+1) N words
 void launch_matmult_loop(he_ctx *ctx, const he_ptmat *pm, int r, int c, const uint64_t *ct, const uint64_t *D,
                          uint64_t *acc /*[2][ext][N]*/, uint64_t *cacc /*[2][level+1][N]*/, int accumulate);
+
+void launch_matmult_rows(he_ctx *ctx, const he_ptmat *pm, int r, int c, const uint64_t *ct, const uint64_t *D, uint64_t *acc /*[2][2][ext][N]*/,
+                         int accumulate);
+bool mm_rows_fit(const he_ctx *ctx, const he_ptmat *pm);
 
 void launch_matmult_loop_with_tables(he_ctx *ctx, const he_ptmat *pm, int r, int c, const uint64_t *ct, const uint64_t *D,
                                      const uint64_t *const *keys, const uint32_t *galois, uint64_t *acc, uint64_t *cacc, int accumulate);

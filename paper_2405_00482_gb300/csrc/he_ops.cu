@@ -1279,6 +1279,166 @@ __global__ void __launch_bounds__(256) fuse_keys_kernel(const uint64_t *__restri
     }
 }
 
+// ---- several row blocks of one MatMult at once ----
+// The row blocks of a product rotate the same ciphertext with the same keys: only their plaintexts
+// differ.  This form runs ROWS of them in one launch, so that a step's key rows are read, multiplied
+// with the digits and reduced once,
+//   t_c = redc(sum_d D[d][u][src] keyM[d][c] (+ c0[u][src] PM for c = 0, u < nq)),   acc_{r,c} += t_c ptM_r,
+// PM the Montgomery form of P mod q_u: a term P x of the accumulator becomes exactly x in ModDown, so
+// the c0 part needs no accumulator of its own, nor does step 0, which is added as P c0 pt and P c1 pt.
+// Sums mod q of the same terms, so the rescaled ciphertexts are those of matmult_loop_kernel.
+// The tile is that of loop variant 5 (16-byte copies into private stages, gathers too).  Two rows are
+// what 128 registers hold (two CTAs of 7-8 warps per multiprocessor); a step of two row blocks costs 11
+// 128-bit multiply-adds and 2 reductions instead of 18 and 4.  N = 2^13, 4 extended limbs, 3 digits, 511
+// rotations: 243 us for two row blocks (1.07 GB read, 4.4 TB/s, 46% of the issue slots: bound by the
+// multiply-adds' latency at 14 warps), where variant 5 takes 2 x 202 us and its fused-key form, which
+// has fewer operations but reads 6 limbs per row block and step, 2 x 149 us.
+constexpr int MMR_G = 4, MMR_S = 2, MMR_VEC = 2;
+template <int ND, int ROWS>
+constexpr int MMR_FIELDS = 3 * ND + ROWS + 1;
+template <int ND, int ROWS>
+constexpr size_t MMR_BYTES = (size_t)MMR_S *MMR_FIELDS<ND, ROWS> *MM_THREADS *MMR_VEC * sizeof(uint64_t);
+struct MMRowsConst {
+    uint64_t pm[HE_MAX_Q];  // P 2^64 mod q_u
+};
+
+template <int ND, int ROWS>
+__global__ void __launch_bounds__(MM_THREADS, 2) matmult_rows_kernel(const uint64_t *ct, const uint64_t *D, const uint64_t *pts, int64_t row_words,
+                                                                     const uint64_t *const *keys, const uint32_t *galois, int m_prime, int ext,
+                                                                     int nq, int L, int LK, uint64_t *acc, int accumulate,
+                                                                     const __grid_constant__ MMRowsConst rcst, const ModConst *__restrict__ mc, int logn) {
+    constexpr int VEC = MMR_VEC, G = MMR_G, SP = MMR_S, F = MMR_FIELDS<ND, ROWS>;
+    constexpr int FP = 2 * ND, FG = FP + ROWS, FC = FG + ND;  // fields: keys, plaintexts, digit gathers, c0 gather
+    HE_GRID_DEP();
+    __shared__ MMTables tb;
+    extern __shared__ uint4 mm_pipe[];
+    uint64_t *pipe = reinterpret_cast<uint64_t *>(mm_pipe);
+    const uint64_t *const *k_use;
+    const uint32_t *g_use;
+    stage_tables(tb, keys, galois, m_prime, k_use, g_use);
+    const int N = 1 << logn, per_limb = N / VEC, lanes = (int)blockDim.x / G;
+    const int lane = (int)threadIdx.x % lanes, grp = (int)threadIdx.x / lanes;
+    const int flat = (int)blockIdx.x * lanes + lane;
+    const bool live = flat / per_limb < ext;  // lanes past the last limb only synchronise
+    const int u = live ? flat / per_limb : 0, k = (flat % per_limb) * VEC;
+    const bool inq = u < nq;
+    const int kl = inq ? u : L + (u - nq);
+    const uint64_t q = mc[kl].q, qinv = mc[kl].qinv, pm = inq ? rcst.pm[u] : 0;
+
+    uint64_t r[ROWS][2][VEC];
+#pragma unroll
+    for (int a = 0; a < ROWS; ++a)
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) r[a][0][j] = r[a][1][j] = 0;
+    if (live) {
+        u128 t[ROWS][2][VEC];
+#pragma unroll
+        for (int a = 0; a < ROWS; ++a)
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) t[a][0][j] = t[a][1][j] = 0;
+        const int period = lazy_terms(q);
+        int pending = 0;
+        uint32_t odd_bits = 0;  // bit st: the parity of the gather source staged in stage st
+        auto slot = [&](int st, int f) { return pipe + ((st * F + f) * MM_THREADS + (int)threadIdx.x) * VEC; };
+        auto issue = [&](int step) {
+            const int i = 1 + grp + step * G;
+            if (i < m_prime) {
+                const int st = step % SP;
+                const uint64_t *key = k_use[i - 1] + (int64_t)kl * N + k;
+#pragma unroll
+                for (int f = 0; f < 2 * ND; ++f) cp_async<8 * VEC>(slot(st, f), key + (int64_t)f * LK * N);
+#pragma unroll
+                for (int a = 0; a < ROWS; ++a) cp_async<8 * VEC>(slot(st, FP + a), pts + a * row_words + ((int64_t)i * ext + u) * N + k);
+                const uint32_t src = automorph_src(k, g_use[i - 1], logn), sa = src & ~1u;
+                odd_bits = (odd_bits & ~(1u << st)) | ((src & 1u) << st);
+#pragma unroll
+                for (int d = 0; d < ND; ++d) cp_async<8 * VEC>(slot(st, FG + d), D + ((int64_t)d * ext + u) * N + sa);
+                if (inq) cp_async<8 * VEC>(slot(st, FC), ct + (int64_t)u * N + sa);
+            }
+            cp_async_commit();
+        };
+        auto flush = [&] {
+#pragma unroll
+            for (int a = 0; a < ROWS; ++a)
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int j = 0; j < VEC; ++j) {
+                        r[a][c][j] = add_mod(r[a][c][j], fold(t[a][c][j], q, qinv), q);
+                        t[a][c][j] = 0;
+                    }
+            pending = 0;
+        };
+#pragma unroll
+        for (int step = 0; step < SP; ++step) issue(step);
+        for (int step = 0; 1 + grp + step * G < m_prime; ++step) {
+            cp_async_wait<SP - 1>();
+            const int st = step % SP;
+            // the staged aligned pair holds (src, src ^ 1) in ascending order
+            const int odd = (int)((odd_bits >> st) & 1u);
+            u128 s[2][VEC];
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) {
+                s[0][j] = inq ? (u128)slot(st, FC)[j ^ odd] * pm : 0;
+                s[1][j] = 0;
+            }
+#pragma unroll
+            for (int d = 0; d < ND; ++d)
+#pragma unroll
+                for (int j = 0; j < VEC; ++j) {
+                    const uint64_t dv = slot(st, FG + d)[j ^ odd];
+                    s[0][j] += (u128)dv * slot(st, 2 * d)[j];
+                    s[1][j] += (u128)dv * slot(st, 2 * d + 1)[j];
+                }
+            uint64_t pv[ROWS][VEC];
+#pragma unroll
+            for (int a = 0; a < ROWS; ++a)
+#pragma unroll
+                for (int j = 0; j < VEC; ++j) pv[a][j] = slot(st, FP + a)[j];
+            issue(step + SP);
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+                for (int j = 0; j < VEC; ++j) {
+                    const uint64_t v = fold(s[c][j], q, qinv);
+#pragma unroll
+                    for (int a = 0; a < ROWS; ++a) t[a][c][j] += (u128)v * pv[a][j];
+                }
+            if (++pending == period) flush();
+        }
+        cp_async_wait<0>();
+        flush();
+    }
+    // the groups' sums through the (drained) stages; group g finishes accumulator g = (row, component)
+    __syncthreads();
+    auto R = [&](int g, int o, int j) -> uint64_t & { return pipe[((g * 2 * ROWS + o) * VEC + j) * lanes + lane]; };
+#pragma unroll
+    for (int o = 0; o < 2 * ROWS; ++o)
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) R(grp, o, j) = r[o / 2][o % 2][j];
+    __syncthreads();
+    static_assert(2 * ROWS <= G, "one group per accumulator");
+    if (!live || grp >= 2 * ROWS) return;
+    const int a = grp / 2, c = grp % 2;
+    uint64_t v[VEC];
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) {
+        v[j] = R(0, grp, j);
+        for (int g = 1; g < G; ++g) v[j] = add_mod(v[j], R(g, grp, j), q);
+    }
+    if (inq) {  // i = 0: no rotation
+        const uint64_t *x = ct + ((int64_t)c * nq + u) * N + k, *p0 = pts + a * row_words + (int64_t)u * N + k;
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) v[j] = add_mod(v[j], mont_mul(mont_mul(x[j], pm, q, qinv), p0[j], q, qinv), q);
+    }
+    uint64_t *A = acc + ((int64_t)(a * 2 + c) * ext + u) * N + k;
+    if (accumulate) {
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) v[j] = add_mod(A[j], v[j], q);
+    }
+    stv<VEC>(A, v);
+}
+
 // batch: persistent CTAs pull (tile, limb, job) items from an ordered queue
 template <int NDIG, int VEC, int G, int S, bool GA>
 __global__ void __launch_bounds__(MM_THREADS, VEC == 2 ? 2 : 3) matmult_batch_loop_kernel(
@@ -1379,6 +1539,15 @@ void mm_dispatch(int v, int ndig, F &&f) {
         case 6: mm_dispatch_nd<1, 4, 2, true>(ndig, f); break;
         case 7: mm_dispatch_nd<1, 8, 2, true>(ndig, f); break;
         default: mm_dispatch_nd<2, 4, 0, false>(ndig, f); break;
+    }
+}
+
+template <typename F>
+void mm_rows_dispatch(int ndig, F &&f) {
+    switch (ndig) {
+        case 1: f.template operator()<1>(); break;
+        case 2: f.template operator()<2>(); break;
+        default: f.template operator()<3>(); break;
     }
 }
 
@@ -1694,22 +1863,67 @@ void launch_matmult_loop(he_ctx *ctx, const he_ptmat *pm, int r, int c, const ui
     if (ev) cudaEventRecord(ev[1], ctx->stream);
 }
 
-// best of three timed launches (after one untimed) of variant v on block (0, 0); 1e30 on error
-static float time_loop_variant(he_ctx *ctx, he_ptmat *pm, int v, const uint64_t *ct, const uint64_t *D, uint64_t *acc, uint64_t *cacc,
-                               const uint64_t *fused, cudaEvent_t a, cudaEvent_t b) {
+// the rows form, on row blocks r, r + 1 of column block c: acc [2][2][ext][N]
+void launch_matmult_rows(he_ctx *ctx, const he_ptmat *pm, int r, int c, const uint64_t *ct, const uint64_t *D, uint64_t *acc, int accumulate) {
     const ModUpConst &mu = ctx->modup[pm->level];
+    const he_plan &p = pm->plan;
+    const int64_t block = p.m_prime * pm->ext * ctx->n, total = (int64_t)mu.ext * (ctx->n / MMR_VEC);
+    const int lanes = mm_block_lanes(5, total, ctx->sms);  // variant 5 has the same lanes and groups
+    MMRowsConst rc{};
+    for (int j = 0; j <= pm->level; ++j) {
+        const uint64_t q = ctx->primes[j];
+        uint64_t v = ctx->mc[j].r1;
+        for (int i = 0; i < ctx->K; ++i) v = (uint64_t)((u128)v * (ctx->primes[ctx->L + i] % q) % q);
+        rc.pm[j] = v;
+    }
+    cudaEvent_t *ev = prof_pair(ctx, HE_PROF_LOOP);
+    if (ev) cudaEventRecord(ev[0], ctx->stream);
+    ctx->launches++;
+    mm_rows_dispatch(mu.ndig, [&]<int ND>() {
+        launch_k(matmult_rows_kernel<ND, 2>, (unsigned)((total + lanes - 1) / lanes), (unsigned)(lanes * MMR_G), MMR_BYTES<ND, 2>, ctx->stream, ct,
+                 D, (const uint64_t *)pm->data + ((int64_t)r * p.col_blocks + c) * block, p.col_blocks * block, (const uint64_t *const *)pm->d_keys,
+                 (const uint32_t *)pm->d_galois, (int)p.m_prime, mu.ext, pm->level + 1, ctx->L, ctx->L + ctx->K, acc, accumulate, rc,
+                 (const ModConst *)ctx->d_mc, ctx->log_n);
+    });
+    if (ev) cudaEventRecord(ev[1], ctx->stream);
+}
+
+// Row blocks in pairs: two or more of them, rotations to share, and one to three digits.  Faster than one
+// by one over the whole range of sizes (a product of two row blocks, the fastest variant one by one ->
+// in pairs): N = 2^13, m' = 2: 51.6 -> 45.6 us, 64: 105 -> 79, 512: 446 -> 287; N = 2^12, m' = 64: 58.4 ->
+// 57.6; N = 2^14, m' = 64: 431 -> 310.  The fused-key form is used only where it beats the pair's time.
+bool mm_rows_fit(const he_ctx *ctx, const he_ptmat *pm) {
+    const int nd = ctx->modup[pm->level].ndig;
+    return pm->plan.row_blocks >= 2 && pm->plan.m_prime > 1 && !pm->plan.baby && nd >= 1 && nd <= 3;
+}
+
+// best of three timed launches (after one untimed) of `go`, of one if that already took longer than
+// `limit`; 1e30 on error
+template <typename F>
+static float time_loop(he_ctx *ctx, cudaEvent_t a, cudaEvent_t b, float limit, F &&go) {
     float ms = 1e30f;
     for (int rep = 0; rep < 4; ++rep) {
         cudaEventRecord(a, ctx->stream);
-        mm_launch_variant(ctx, v, ct, D, pm->data, pm->d_keys, pm->d_galois, (int)pm->plan.m_prime, mu.ndig, mu.ext, pm->level + 1, acc, cacc, 0,
-                          fused);
+        go();
         cudaEventRecord(b, ctx->stream);
         if (cudaEventSynchronize(b) != cudaSuccess) break;
         float t = 0.0f;
         cudaEventElapsedTime(&t, a, b);
         if (rep > 0 && t < ms) ms = t;
+        if (ms < 1e30f && ms > limit) break;
     }
     return ms;
+}
+
+// variant v on block (0, 0), next to the fastest so far (`best`): a launch takes the same time within
+// a few percent, so one that is a quarter slower is not timed again
+static float time_loop_variant(he_ctx *ctx, he_ptmat *pm, int v, const uint64_t *ct, const uint64_t *D, uint64_t *acc, uint64_t *cacc,
+                               const uint64_t *fused, cudaEvent_t a, cudaEvent_t b, float best) {
+    const ModUpConst &mu = ctx->modup[pm->level];
+    return time_loop(ctx, a, b, 1.25f * best, [&] {
+        mm_launch_variant(ctx, v, ct, D, pm->data, pm->d_keys, pm->d_galois, (int)pm->plan.m_prime, mu.ndig, mu.ext, pm->level + 1, acc, cacc, 0,
+                          fused);
+    });
 }
 
 // Time the fused-key forms of the staged variants on this matrix (its tables built) and keep the
@@ -1726,7 +1940,7 @@ int tune_matmult_fused(he_ctx *ctx, he_ptmat *pm, const uint64_t *ct, const uint
     for (int v = 0; v < mm_variant_count(); ++v) {
         pm->fuse_ms[v] = 0.0f;
         if (!mm_variant_fusable(v, ndig)) continue;
-        pm->fuse_ms[v] = time_loop_variant(ctx, pm, v, ct, D, acc, cacc, pm->fused, a, b);
+        pm->fuse_ms[v] = time_loop_variant(ctx, pm, v, ct, D, acc, cacc, pm->fused, a, b, best < 0 ? 1e30f : pm->fuse_ms[best]);
         if (best < 0 || pm->fuse_ms[v] < pm->fuse_ms[best]) best = v;
     }
     cudaEventDestroy(a);
@@ -1737,7 +1951,7 @@ int tune_matmult_fused(he_ctx *ctx, he_ptmat *pm, const uint64_t *ct, const uint
 
 // Time every loop-kernel variant once on this matrix's first product (the results are identical:
 // modular sums do not depend on the order) and keep the fastest.  Synchronises the stream.
-int tune_matmult_loop(he_ctx *ctx, he_ptmat *pm, const uint64_t *ct, const uint64_t *D, uint64_t *acc, uint64_t *cacc) {
+int tune_matmult_loop(he_ctx *ctx, he_ptmat *pm, const uint64_t *ct, const uint64_t *D, uint64_t *acc, uint64_t *cacc, bool rows) {
     cudaEvent_t a, b;
     if (cudaEventCreate(&a) != cudaSuccess) return HE_ECUDA;
     if (cudaEventCreate(&b) != cudaSuccess) {
@@ -1747,14 +1961,15 @@ int tune_matmult_loop(he_ctx *ctx, he_ptmat *pm, const uint64_t *ct, const uint6
     int best = 0;
     float best_ms = 1e30f;
     for (int v = 0; v < mm_variant_count(); ++v) {
-        // one untimed launch (it also loads the variant's code), then the best of three
-        const float ms = time_loop_variant(ctx, pm, v, ct, D, acc, cacc, nullptr, a, b);
+        // one untimed launch (it also loads the variant's code), then the best of up to three
+        const float ms = time_loop_variant(ctx, pm, v, ct, D, acc, cacc, nullptr, a, b, best_ms);
         pm->tune_ms[v] = ms;
         if (ms < best_ms) {
             best_ms = ms;
             best = v;
         }
     }
+    if (rows) pm->rows_ms = time_loop(ctx, a, b, 0.0f, [&] { launch_matmult_rows(ctx, pm, 0, 0, ct, D, acc, 0); });
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     pm->variant = best;
@@ -1939,6 +2154,11 @@ void ops_set_smem_limits(int max_bytes) {
     });
     each_logn([max_bytes](auto L) { cudaFuncSetAttribute(moddown_rescale_intt_kernel<L.value>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes); });
     each_logn([max_bytes](auto L) { cudaFuncSetAttribute(moddown_rescale_ntt_kernel<L.value>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes); });
+    for (int nd = 1; nd <= 3; ++nd)
+        mm_rows_dispatch(nd, []<int ND>() {
+            cudaFuncSetAttribute(matmult_rows_kernel<ND, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MMR_BYTES<ND, 2>);
+            cudaFuncSetAttribute(matmult_rows_kernel<ND, 2>, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        });
 
     for (int v = 0; v < kMMVariants; ++v)
         for (int nd = 0; nd <= 3; ++nd)
