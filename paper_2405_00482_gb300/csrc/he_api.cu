@@ -1129,6 +1129,8 @@ int ptmat_bind_keys(he_ctx *ctx, he_ptmat *pm) {
     if (cudaMalloc(&pm->d_galois, steps * sizeof(uint32_t)) != cudaSuccess) return HE_ENOMEM;
     if (cudaMemcpy(pm->d_keys, ptrs.data(), steps * sizeof(uint64_t *), cudaMemcpyHostToDevice) != cudaSuccess) return HE_ECUDA;
     if (cudaMemcpy(pm->d_galois, gal.data(), steps * sizeof(uint32_t), cudaMemcpyHostToDevice) != cudaSuccess) return HE_ECUDA;
+    // a copy from pageable memory returns once it is staged: the tables are on the device after this
+    if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) return HE_ECUDA;
     pm->galois = gal;
     return HE_OK;
 }

@@ -1232,14 +1232,19 @@ template <int NDIG, int VEC, int G, int S, bool GA, bool FK = false>
 __global__ void __launch_bounds__(MM_THREADS, VEC == 2 ? 2 : 3) matmult_loop_kernel(
     const uint64_t *__restrict__ ct, const uint64_t *__restrict__ D, const uint64_t *__restrict__ pts,
     const uint64_t *const *__restrict__ keys, const uint32_t *__restrict__ galois, int m_prime, int ndig_rt, int ext, int nq, int L,
-    int LK, uint64_t *acc, uint64_t *cacc, int accumulate, const ModConst *__restrict__ mc, int logn, const uint64_t *__restrict__ fused) {
-    HE_GRID_DEP();
+    int LK, uint64_t *acc, uint64_t *cacc, int accumulate, const ModConst *__restrict__ mc, int logn, const uint64_t *__restrict__ fused,
+    int tables_ready) {
+    HE_GRID_LAUNCH();
     __shared__ uint64_t red[G * 3 * VEC * (MM_THREADS / G)];
     __shared__ MMTables tb;
     extern __shared__ uint4 mm_pipe[];
     const uint64_t *const *k_use;
     const uint32_t *g_use;
-    stage_tables(tb, keys, galois, m_prime, k_use, g_use);
+    // a matrix's own tables are host copies that were complete before this launch: staged while the
+    // previous kernel drains; tables that a kernel writes, only after the wait
+    if (tables_ready) stage_tables(tb, keys, galois, m_prime, k_use, g_use);
+    HE_GRID_WAIT();
+    if (!tables_ready) stage_tables(tb, keys, galois, m_prime, k_use, g_use);
     const int lanes = (int)blockDim.x / G, per_limb = (1 << logn) / VEC;
     const int flat = (int)blockIdx.x * lanes + (int)threadIdx.x % lanes;
     int u = flat / per_limb, k = (flat % per_limb) * VEC;
@@ -1309,13 +1314,14 @@ __global__ void __launch_bounds__(MM_THREADS, 2) matmult_rows_kernel(const uint6
                                                                      const __grid_constant__ MMRowsConst rcst, const ModConst *__restrict__ mc, int logn) {
     constexpr int VEC = MMR_VEC, G = MMR_G, SP = MMR_S, F = MMR_FIELDS<ND, ROWS>;
     constexpr int FP = 2 * ND, FG = FP + ROWS, FC = FG + ND;  // fields: keys, plaintexts, digit gathers, c0 gather
-    HE_GRID_DEP();
+    HE_GRID_LAUNCH();
     __shared__ MMTables tb;
     extern __shared__ uint4 mm_pipe[];
     uint64_t *pipe = reinterpret_cast<uint64_t *>(mm_pipe);
     const uint64_t *const *k_use;
     const uint32_t *g_use;
-    stage_tables(tb, keys, galois, m_prime, k_use, g_use);
+    stage_tables(tb, keys, galois, m_prime, k_use, g_use);  // before the wait: see matmult_loop_kernel
+    HE_GRID_WAIT();
     const int N = 1 << logn, per_limb = N / VEC, lanes = (int)blockDim.x / G;
     const int lane = (int)threadIdx.x % lanes, grp = (int)threadIdx.x / lanes;
     const int flat = (int)blockIdx.x * lanes + lane;
@@ -1574,7 +1580,7 @@ int mm_block_lanes(int v, int64_t total_lanes, int sms) {
 
 void mm_launch_variant(he_ctx *ctx, int v, const uint64_t *ct, const uint64_t *D, const uint64_t *pts, const uint64_t *const *keys,
                        const uint32_t *galois, int m_prime, int ndig, int ext, int nq, uint64_t *acc, uint64_t *cacc, int accumulate,
-                       const uint64_t *fused) {
+                       const uint64_t *fused, bool tables_ready) {
     const int64_t total = (int64_t)ext * (ctx->n / kMMShapes[v].vec);
     const int lanes = mm_block_lanes(v, total, ctx->sms);
     const unsigned grid = (unsigned)((total + lanes - 1) / lanes), threads = (unsigned)(lanes * kMMShapes[v].grp);
@@ -1582,13 +1588,13 @@ void mm_launch_variant(he_ctx *ctx, int v, const uint64_t *ct, const uint64_t *D
     if (fused && mm_variant_fusable(v, ndig)) {
         mm_dispatch_fk(v, ndig, [&]<int NDIG, int VEC, int G, int S, bool GA>() {
             launch_k(matmult_loop_kernel<NDIG, VEC, G, S, GA, true>, grid, threads, mm_pipe_bytes(NDIG, VEC, S, GA), ctx->stream, ct, D, pts, keys,
-                     galois, m_prime, ndig, ext, nq, ctx->L, ctx->L + ctx->K, acc, cacc, accumulate, ctx->d_mc, ctx->log_n, fused);
+                     galois, m_prime, ndig, ext, nq, ctx->L, ctx->L + ctx->K, acc, cacc, accumulate, ctx->d_mc, ctx->log_n, fused, (int)tables_ready);
         });
         return;
     }
     mm_dispatch(v, ndig, [&]<int NDIG, int VEC, int G, int S, bool GA>() {
         launch_k(matmult_loop_kernel<NDIG, VEC, G, S, GA>, grid, threads, mm_pipe_bytes(NDIG, VEC, S, GA), ctx->stream, ct, D, pts, keys, galois,
-                 m_prime, ndig, ext, nq, ctx->L, ctx->L + ctx->K, acc, cacc, accumulate, ctx->d_mc, ctx->log_n, (const uint64_t *)nullptr);
+                 m_prime, ndig, ext, nq, ctx->L, ctx->L + ctx->K, acc, cacc, accumulate, ctx->d_mc, ctx->log_n, (const uint64_t *)nullptr, (int)tables_ready);
     });
 }
 
@@ -1859,7 +1865,7 @@ void launch_matmult_loop(he_ctx *ctx, const he_ptmat *pm, int r, int c, const ui
     cudaEvent_t *ev = prof_pair(ctx, HE_PROF_LOOP);
     if (ev) cudaEventRecord(ev[0], ctx->stream);
     mm_launch_variant(ctx, fk ? pm->fvariant : (pm->variant < 0 ? 0 : pm->variant), ct, D, pts, pm->d_keys, pm->d_galois, (int)p.m_prime,
-                      mu.ndig, mu.ext, level + 1, acc, cacc, accumulate, fused);
+                      mu.ndig, mu.ext, level + 1, acc, cacc, accumulate, fused, true);
     if (ev) cudaEventRecord(ev[1], ctx->stream);
 }
 
@@ -1922,7 +1928,7 @@ static float time_loop_variant(he_ctx *ctx, he_ptmat *pm, int v, const uint64_t 
     const ModUpConst &mu = ctx->modup[pm->level];
     return time_loop(ctx, a, b, 1.25f * best, [&] {
         mm_launch_variant(ctx, v, ct, D, pm->data, pm->d_keys, pm->d_galois, (int)pm->plan.m_prime, mu.ndig, mu.ext, pm->level + 1, acc, cacc, 0,
-                          fused);
+                          fused, true);
     });
 }
 
@@ -1985,7 +1991,7 @@ void launch_matmult_loop_with_tables(he_ctx *ctx, const he_ptmat *pm, int r, int
     const he_plan &p = pm->plan;
     const uint64_t *pts = pm->data + (((int64_t)r * p.col_blocks + c) * p.m_prime) * pm->ext * ctx->n;
     mm_launch_variant(ctx, pm->variant < 0 ? 0 : pm->variant, ct, D, pts, keys, galois, (int)p.m_prime, mu.ndig, mu.ext, level + 1, acc, cacc,
-                      accumulate, nullptr);
+                      accumulate, nullptr, false);
 }
 
 void launch_layout_matrix(he_ctx *ctx, const he_plan &p, const double *X, double *slots, int trans) {
