@@ -830,6 +830,13 @@ __device__ __forceinline__ void ldv(const uint64_t *p, uint64_t (&o)[VEC]) {
 }
 // gather of VEC values at the automorphism image of k..k+VEC-1 (src of k given)
 template <int VEC>
+__device__ __forceinline__ void ldv(const uint64_t *p, uint64_t (&o)[VEC], uint64_t policy) {
+    if constexpr (VEC == 2)
+        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.u64 {%0, %1}, [%2], %3;" : "=l"(o[0]), "=l"(o[1]) : "l"(p), "l"(policy));
+    else
+        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u64 %0, [%1], %2;" : "=l"(o[0]) : "l"(p), "l"(policy));
+}
+template <int VEC>
 __device__ __forceinline__ void gatherv(const uint64_t *base, uint32_t src, uint64_t (&o)[VEC]) {
     if constexpr (VEC == 2) {
         const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(base + (src & ~1u));
@@ -859,6 +866,20 @@ __device__ __forceinline__ void cp_async(uint64_t *smem, const uint64_t *gmem) {
     else
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
+// an L2 replacement hint for streamed data: its lines give way before those of the usual priority
+__device__ __forceinline__ uint64_t l2_evict_first() {
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+template <int BYTES>
+__device__ __forceinline__ void cp_async(uint64_t *smem, const uint64_t *gmem, uint64_t policy) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "l"(policy) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 8, %2;\n" ::"r"(sa), "l"(gmem), "l"(policy) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int PENDING>
 __device__ __forceinline__ void cp_async_wait() {
@@ -881,7 +902,16 @@ __device__ __forceinline__ void cp_async_wait() {
 // the same residue as the two-level form: no per-step reduction and no second product.  The
 // 128-bit sums then take up to 2^(128 - 2 bits(q)) products (64 for q < 2^61); their high word is
 // reduced mod q before the Montgomery step, whose input must stay below q 2^64.
-template <int NDIG, int VEC, int G, int S, bool GA, bool FK = false>
+//
+// With KH (the single product) the key operands, fused or not, are read with L2 evict_first.  A
+// matrix's keys or tables (100 MB at N = 2^13, m' = 64) and its plaintexts just exceed the 129 MB cache:
+// read in the same order by every call with the usual priority, each line was gone when its turn came
+// again, and the freshly encoded plaintexts were written back to memory to make room (97 MB read and
+// 19-30 MB written in the loop of an encode, encrypt, multiply, decrypt step; by physical placement
+// 157-163 us a step).  Giving way first, most of the stream stays and nothing else is pushed out: 140.5 us
+// whatever the placement, 1024 x 256 with fused tables 51.5 -> 48.0.  The batch reads a key for many jobs
+// and loses 1.4% by a hint; streams far above the cache (row pairs, key switch) gain nothing.
+template <int NDIG, int VEC, int G, int S, bool GA, bool FK, bool KH>
 __device__ __forceinline__ void mm_tile(const uint64_t *__restrict__ ct, const uint64_t *__restrict__ D, const uint64_t *__restrict__ pts,
                                         const uint64_t *const *keys, const uint32_t *galois, int m_prime,
                                         int ndig_rt, int ext, int nq, int L, int LK, int u, int k, int lanes, uint64_t *acc,
@@ -895,6 +925,19 @@ __device__ __forceinline__ void mm_tile(const uint64_t *__restrict__ ct, const u
     const bool inq = u < nq;
     const int lane = threadIdx.x % lanes, grp = threadIdx.x / lanes;
     auto R = [&](int g, int which, int j) -> uint64_t & { return red[((g * 3 + which) * VEC + j) * lanes + lane]; };
+    const uint64_t kpol = KH ? l2_evict_first() : 0;
+    auto key_async = [&](uint64_t *smem, const uint64_t *gmem) {
+        if constexpr (KH)
+            cp_async<8 * VEC>(smem, gmem, kpol);
+        else
+            cp_async<8 * VEC>(smem, gmem);
+    };
+    auto key_load = [&](const uint64_t *gmem, uint64_t (&o)[VEC]) {
+        if constexpr (KH)
+            ldv<VEC>(gmem, o, kpol);
+        else
+            ldv<VEC>(gmem, o);
+    };
 
     uint64_t r0[VEC], r1[VEC], rc[VEC];
 #pragma unroll
@@ -929,14 +972,14 @@ __device__ __forceinline__ void mm_tile(const uint64_t *__restrict__ ct, const u
                     if constexpr (FK) {
                         const uint64_t *f = fused + ((int64_t)(i - 1) * 2 * ND * ext + u) * N + k;
 #pragma unroll
-                        for (int d = 0; d < 2 * ND; ++d) cp_async<8 * VEC>(slot(st, d), f + (int64_t)d * ext * N);
+                        for (int d = 0; d < 2 * ND; ++d) key_async(slot(st, d), f + (int64_t)d * ext * N);
                         if (inq) cp_async<8 * VEC>(slot(st, 2 * ND), pts + ((int64_t)i * ext + u) * N + k);
                     } else {
                         const uint64_t *key = keys[i - 1];
 #pragma unroll
                         for (int d = 0; d < ND; ++d) {
-                            cp_async<8 * VEC>(slot(st, 2 * d), key + ((int64_t)(d * 2 + 0) * LK + kl) * N + k);
-                            cp_async<8 * VEC>(slot(st, 2 * d + 1), key + ((int64_t)(d * 2 + 1) * LK + kl) * N + k);
+                            key_async(slot(st, 2 * d), key + ((int64_t)(d * 2 + 0) * LK + kl) * N + k);
+                            key_async(slot(st, 2 * d + 1), key + ((int64_t)(d * 2 + 1) * LK + kl) * N + k);
                         }
                         cp_async<8 * VEC>(slot(st, 2 * ND), pts + ((int64_t)i * ext + u) * N + k);
                     }
@@ -1083,8 +1126,8 @@ __device__ __forceinline__ void mm_tile(const uint64_t *__restrict__ ct, const u
                 for (int d = 0; d < ND; ++d) {
                     if (NDIG == 0 && d >= ndig) break;
                     gatherv<VEC>(D + ((int64_t)d * ext + u) * N, src, dv[d]);
-                    ldv<VEC>(key + ((int64_t)(d * 2 + 0) * LK + kl) * N + k, kv0[d]);
-                    ldv<VEC>(key + ((int64_t)(d * 2 + 1) * LK + kl) * N + k, kv1[d]);
+                    key_load(key + ((int64_t)(d * 2 + 0) * LK + kl) * N + k, kv0[d]);
+                    key_load(key + ((int64_t)(d * 2 + 1) * LK + kl) * N + k, kv1[d]);
                 }
                 ldv<VEC>(pts + ((int64_t)i * ext + u) * N + k, pm);
                 if (inq) gatherv<VEC>(ct + (int64_t)u * N, src, cv);
@@ -1252,7 +1295,7 @@ __global__ void __launch_bounds__(MM_THREADS, VEC == 2 ? 2 : 3) matmult_loop_ker
         u = 0;
         k = 1 << logn;
     }
-    mm_tile<NDIG, VEC, G, S, GA, FK>(ct, D, pts, k_use, g_use, m_prime, ndig_rt, ext, nq, L, LK, u, k, lanes, acc, cacc, accumulate, mc, logn,
+    mm_tile<NDIG, VEC, G, S, GA, FK, true>(ct, D, pts, k_use, g_use, m_prime, ndig_rt, ext, nq, L, LK, u, k, lanes, acc, cacc, accumulate, mc, logn,
                                      red, reinterpret_cast<uint64_t *>(mm_pipe), fused);
 }
 
@@ -1473,7 +1516,7 @@ __global__ void __launch_bounds__(MM_THREADS, VEC == 2 ? 2 : 3) matmult_batch_lo
         const uint32_t *g_use;
         stage_tables(tb, jb.keys, jb.galois, jb.m_prime, k_use, g_use);
         constexpr int LANES = MM_THREADS / G;
-        mm_tile<NDIG, VEC, G, S, GA>(jb.ct, bg.D + (int64_t)j * bg.d_words, jb.pts, k_use, g_use, jb.m_prime, bg.ndig, bg.ext, bg.nq, bg.L,
+        mm_tile<NDIG, VEC, G, S, GA, false, false>(jb.ct, bg.D + (int64_t)j * bg.d_words, jb.pts, k_use, g_use, jb.m_prime, bg.ndig, bg.ext, bg.nq, bg.L,
                                      bg.LK, u, tile * TILE + VEC * ((int)threadIdx.x % LANES), LANES, bg.acc + (int64_t)j * bg.acc_words,
                                      bg.cacc + (int64_t)j * bg.cacc_words, 0, mc, logn, red, reinterpret_cast<uint64_t *>(mm_pipe));
         __syncthreads();
