@@ -651,6 +651,7 @@ int he_encrypt_dnonce(he_ctx *ctx, const he_pt *pt, const uint64_t *nonce_dev, h
 int he_decrypt(he_ctx *ctx, const he_ct *ct, double *slots_out) {
     if (!ctx || !ct || !ct->data || !slots_out) return HE_EINVAL;
     if (ct->level < 0 || ct->level >= ctx->L) return HE_ELEVEL;
+    if (launch_decrypt_slots(ctx, ct, slots_out)) return last_launch();
     double *coef = reinterpret_cast<double *>(ctx_scratch(ctx, ctx->n));
     if (!coef) return HE_ENOMEM;
     launch_decrypt_coeffs(ctx, ct->data, ct->level, 1, coef, nullptr);
@@ -1513,6 +1514,7 @@ int he_matmult_decrypt(he_ctx *ctx, const he_plan *plan, const he_ct *cts, int n
         if (cts[r].level < 0 || cts[r].level >= ctx->L) return HE_ELEVEL;
         if (cts[r].scale != cts[0].scale) return HE_ESCALE;
     }
+    if (launch_decrypt_ras(ctx, *plan, cts, n_ct, mask, y_out)) return last_launch();
     const size_t N = ctx->n;
     uint64_t *s = ctx_scratch(ctx, (size_t)n_ct * N + (size_t)n_ct * (N / 2));
     if (!s) return HE_ENOMEM;

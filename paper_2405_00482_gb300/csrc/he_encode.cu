@@ -555,6 +555,12 @@ __global__ void encode_pair_cl_kernel(SRC src, int count, double scale, const fl
 // slot values, so the same doubles without the slot array.
 // Each epilogue's slot positions of its first two iterations are read by prefetch() before the
 // kernel waits for its predecessor.
+// the ciphertexts of one fused decryption
+constexpr int HE_DECRYPT_MAX = 16;
+struct DecryptSrc {
+    const uint64_t *ct[HE_DECRYPT_MAX];
+    int32_t nl[HE_DECRYPT_MAX];  // limbs of each component
+};
 struct EpiPre {
     int pos[2];
 };
@@ -717,6 +723,66 @@ __global__ void decrypt_kernel(const uint64_t *__restrict__ ct, int64_t ct_words
         const uint64_t v = mul_shoup(s[SIDX(k)], mc[0].ninv, mc[0].ninv_shoup, q);
         o[k] = v > half ? u64_to_double_rn(q - v, true) : u64_to_double_rn(v, false);
     }
+}
+
+// decrypt_kernel<true> and decode_cl_kernel in one launch, a cluster per ciphertext: each CTA sends the
+// centred coefficients of its slice straight to their bit-reversed places in the cluster's shared
+// memory (stores, which nothing waits for; gathering them instead, with 4-way bank conflicts on loads
+// that everything waits for, cost 1.4 us more at N = 2^14 and was slower than two launches).  A decryption
+// is a chain of barriers in eight CTAs; as two launches it also went through global memory and a kernel
+// boundary.  An encode, encrypt, multiply, decrypt step of 16 x 64 at N = 2^12: 52.1 -> 47.1 us, of
+// 256 x 1024 at N = 2^13: 143.0 -> 141.7; a ciphertext at N = 2^14 22.1 -> 21.6 us.
+// src holds pointers that earlier launches wrote through: read after the wait, no __restrict__.
+template <int LOGN, class EPI>
+__global__ void decrypt_decode_cl_kernel(const __grid_constant__ DecryptSrc src, const uint64_t *__restrict__ sk_mont, double scale,
+                                         const float4 *__restrict__ tw, const float4 *__restrict__ twist, const int32_t *__restrict__ slot_pos, EPI epi,
+                                         const uint64_t *__restrict__ d_tw, const ModConst *__restrict__ mc, int logn_rt) {
+    HE_GRID_LAUNCH();
+    constexpr int CLG = 3;
+    const int logn = LOGN ? LOGN : logn_rt;
+    cg::cluster_group cl = cg::this_cluster();
+    const int logm = logn - 1, M = 1 << logm, lg_ms = logm - CLG, MS = 1 << lg_ms;
+    int item, off, len;
+    slice_of<true>(logn, item, off, len);
+    const int rank = (int)cl.block_rank(), foff = rank * MS;
+    uint64_t *s = s_dyn();  // the slice and its twiddles, then the transform's slice and twiddles
+    float4 *a = reinterpret_cast<float4 *>(s + cl_tw_offset_words(logn) + 2 * len);
+    // the context's tables before the wait, as in the two kernels
+    const ulonglong2 *itw = twiddles(d_tw, 0, 1, logn);
+    tw_prefetch<true, false>(s, itw, logn);
+    fft_tw_issue<CLG>(a, tw, logm);
+    float4 w_pre[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+        if ((int)threadIdx.x + r * (int)blockDim.x < MS) w_pre[r] = twist[__brev(foff + threadIdx.x + r * blockDim.x) >> (32 - logm)];
+    const EpiPre pre = epi.prefetch(item, rank, CLG, M, lg_ms, slot_pos);
+    const uint64_t q = mc[0].q, qinv = mc[0].qinv, ninv = mc[0].ninv, ninvs = mc[0].ninv_shoup, half = q >> 1;
+    HE_GRID_WAIT();
+    const uint64_t *c0 = src.ct[item] + off, *c1 = c0 + ((int64_t)src.nl[item] << logn);
+    for (int k = threadIdx.x; k < len; k += blockDim.x) s[SIDX(k)] = add_mod(c0[k], mont_mul(c1[k], sk_mont[off + k], q, qinv), q);
+    __syncthreads();
+    ntt_inv_cluster<LOGN>(s, itw, q, logn);
+    // coefficient k (and k + M as the imaginary part) goes to its bit-reversed position, in the CTA that holds it
+    for (int k = threadIdx.x; k < len; k += blockDim.x) {
+        const uint64_t v = mul_shoup(s[SIDX(k)], ninv, ninvs, q);
+        const double x = v > half ? u64_to_double_rn(q - v, true) : u64_to_double_rn(v, false);
+        const int t = __brev((off + k) & (M - 1)) >> (32 - logm);
+        reinterpret_cast<double *>(cl.map_shared_rank(a, t >> lg_ms) + (t & (MS - 1)))[off >= M] = x;
+    }
+    cl.sync();
+    int r = 0;
+    for (int i = threadIdx.x; i < MS; i += blockDim.x, ++r) {
+        const float4 w = r == 0 ? w_pre[0] : (r == 1 ? w_pre[1] : twist[__brev(foff + i) >> (32 - logm)]);
+        const double2 z = reinterpret_cast<const double2 *>(a)[i];
+        const df re = df_from(z.x), im = df_from(z.y);
+        float4 c;
+        cmul(make_float4(re.hi, re.lo, im.hi, im.lo), make_float4(w.x, w.y, -w.z, -w.w), c);
+        a[i] = c;
+    }
+    __syncthreads();
+    fft_cluster<CLG, 1, LOGN ? LOGN - 1 : 0>(a, tw, logm, +1);
+    epi(cl, a, item, rank, CLG, M, lg_ms, slot_pos, 1.0 / scale, reinterpret_cast<double *>(a + MS), pre);
+    cl.barrier_wait();  // the epilogue arrived once the other CTAs' shared memory was last read
 }
 
 // ---- Philox-4x64-10 (Salmon et al., SC'11) ----
@@ -1045,12 +1111,16 @@ void launch_decode(he_ctx *ctx, const double *coeffs, int count, double scale, d
     launch_k(decode_kernel, count, FFT_THREADS, fft_smem_bytes(ctx->log_n), ctx->stream, coeffs, scale, tw, twist, pos, slots, ctx->log_n);
 }
 
+static DecodeRas ras_epilogue(const he_plan &p, const double *mask, double *y) {
+    auto lg = [](int64_t v) { return __builtin_ctzll((unsigned long long)v); };
+    return DecodeRas{p, mask, y, lg(p.m_prime), lg(p.nb), lg(p.slots), lg(p.mb)};
+}
+
 bool launch_decode_ras(he_ctx *ctx, const he_plan &p, const double *coeffs, int count, double scale, const double *mask, double *y) {
     const float4 *tw = reinterpret_cast<const float4 *>(ctx->d_fft);
     const float4 *twist = tw + ctx->n / 4;
     const int32_t *pos = reinterpret_cast<const int32_t *>(twist + ctx->n / 2);
-    auto lg = [](int64_t v) { return __builtin_ctzll((unsigned long long)v); };
-    const DecodeRas epi{p, mask, y, lg(p.m_prime), lg(p.nb), lg(p.slots), lg(p.mb)};
+    const DecodeRas epi = ras_epilogue(p, mask, y);
     switch (fft_cluster_log(ctx->log_n, count)) {
         case 3:
             launch_fft_cl<3, 1>(by_logn(ctx->log_n, [](auto L) { return decode_cl_kernel<3, 1, L.value, DecodeRas>; }), ctx, count, coeffs, scale, tw, twist,
@@ -1080,6 +1150,38 @@ void launch_decrypt_coeffs(he_ctx *ctx, const uint64_t *ct, int level, int count
     }
     launch_k(by_logn(ctx->log_n, [](auto L) { return decrypt_kernel<false, L.value>; }), count, ntt_threads(ctx->log_n), ntt_smem_bytes(ctx->log_n), ctx->stream, ct, words, level + 1, ctx->d_sk_mont, coeffs, ctx->d_tw, ctx->d_mc,
                                                                     ctx->log_n);
+}
+
+// decryption and decode of `count` ciphertexts in one launch; false (nothing launched) where the
+// cluster forms of both do not apply or there are more ciphertexts than the launch's table holds
+template <class EPI>
+static bool launch_decrypt_decode(he_ctx *ctx, const he_ct *cts, int count, const EPI &epi) {
+    if (count < 1 || count > HE_DECRYPT_MAX || !use_cluster(ctx->log_n, count) || fft_cluster_log(ctx->log_n, count) != 3) return false;
+    const size_t bytes = cl_smem_bytes(ctx->log_n) + (size_t)(ctx->n / 16) * sizeof(float4) * 3 / 2;
+    DecryptSrc src{};
+    for (int i = 0; i < count; ++i) {
+        src.ct[i] = cts[i].data;
+        src.nl[i] = cts[i].level + 1;
+    }
+    const float4 *tw = reinterpret_cast<const float4 *>(ctx->d_fft);
+    const float4 *twist = tw + ctx->n / 4;
+    ctx->launches++;
+    launch_cluster(by_logn(ctx->log_n, [](auto L) { return decrypt_decode_cl_kernel<L.value, EPI>; }), count * HE_NTT_CL_SIZE, cl_threads(ctx->log_n),
+                   bytes, ctx->stream, src, (const uint64_t *)ctx->d_sk_mont,
+                   cts[0].scale, tw, twist, reinterpret_cast<const int32_t *>(twist + ctx->n / 2), epi, (const uint64_t *)ctx->d_tw,
+                   (const ModConst *)ctx->d_mc, ctx->log_n);
+    return true;
+}
+
+bool launch_decrypt_slots(he_ctx *ctx, const he_ct *ct, double *slots) { return launch_decrypt_decode(ctx, ct, 1, DecodeSlots{slots}); }
+
+bool launch_decrypt_ras(he_ctx *ctx, const he_plan &p, const he_ct *cts, int count, const double *mask, double *y) {
+    // a cluster writes its results while another may still read its ciphertext
+    for (int i = 0; count > 1 && i < count; ++i) {
+        const uintptr_t d = (uintptr_t)cts[i].data, o = (uintptr_t)y;
+        if (o < d + 2 * (size_t)(cts[i].level + 1) * ctx->n * sizeof(uint64_t) && d < o + (size_t)p.m * sizeof(double)) return false;
+    }
+    return launch_decrypt_decode(ctx, cts, count, ras_epilogue(p, mask, y));
 }
 
 void launch_sample_uniform(he_ctx *ctx, uint64_t tag, uint64_t nonce, const LimbMap &map, int, uint64_t *out, const uint64_t *nonce_dev) {
@@ -1140,6 +1242,8 @@ void encode_set_smem_limits(int max_bytes) {
     each_logn([max_bytes](auto L) {
         cudaFuncSetAttribute(decrypt_kernel<false, L.value>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
         cudaFuncSetAttribute(decrypt_kernel<true, L.value>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
+        cudaFuncSetAttribute(decrypt_decode_cl_kernel<L.value, DecodeSlots>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
+        cudaFuncSetAttribute(decrypt_decode_cl_kernel<L.value, DecodeRas>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
         cudaFuncSetAttribute(encrypt_ntt_cl_kernel<L.value>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
         // cluster FFTs: the slice and the local stages' twiddles (1.5 MS float4)
         cudaFuncSetAttribute(encode_cl_kernel<1, 1, L.value, SlotsSrc>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
