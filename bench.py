@@ -556,7 +556,7 @@ BUTTERFLY_INSTR = 28
 def _peaks() -> dict:
     p = os.path.join(ROOT, "MEASURED_PEAKS.json")
     d = json.load(open(p)) if os.path.exists(p) else {}
-    return {"hbm_gbs": float(d.get("hbm_gbs", 6800.0)), "source": "MEASURED_PEAKS.json (measured)" if d else "fallback 6800 GB/s"}
+    return {"hbm_gbs": float(d.get("hbm_gbs", 6800.0)), "bf16_tflops": float(d.get("bf16_tflops", 1900.0)), "source": "MEASURED_PEAKS.json (measured)" if d else "fallback 6800 GB/s, 1900 TFLOP/s bf16"}
 
 
 def _event_times(fn, reps, flush, warm=3):
@@ -743,9 +743,11 @@ def run_vfl_nn(he, inputs, args, flush, world, dev, rank):
     s_fwd = max_over_ranks(sum(t_fwd) / 1e3, world, dev)
     macs = K * (level + 1) * P.n * 2 * n  # 64-bit modular multiply-adds of one forward product
     fwd_ms = statistics.median(t_fwd)
-    # ALU peak: 64 32-bit IMAD per SM per clock x 152 SMs x 2.07 GHz, 4 IMAD per 64x64 -> 128-bit product
-    peak = 64 * 152 * 2.07e9 / 4 / 1e12
-    achieved = macs / (fwd_ms / 1e3) / 1e12
+    # on the tensor cores each multiply-add is one bf16 product per modulus: 10 moduli for the 40-bit
+    # primes' limbs, 15 for the 60-bit one's
+    achieved = macs * (10 * level + 15) / (level + 1) * 2 / (fwd_ms / 1e3) / 1e12
+    peaks = _peaks()
+    peak = peaks["bf16_tflops"]
     return {"workload": "A 4096x256 ~ U[-1,1] as 256 diagonal ciphertexts, W 256x128 ~ N(0,1/256), D^T 4096x128 ~ N(0,1/4096); "
                         "N=16384, Q=[60,40x6], P=[60,60,60], dnum=3, scale 2^40",
             "forward_per_sec": round(whole_job_rate(reps, world, s_fwd), 2), "forward_ms": {"p50": _pct(t_fwd, 0.5), "p99": _pct(t_fwd, 0.99)},
@@ -754,9 +756,10 @@ def run_vfl_nn(he, inputs, args, flush, world, dev, rank):
             "transpose_int8_tc_ms": {"p50": _pct(t_tr8, 0.5), "p99": _pct(t_tr8, 0.99), "basis_extension": "INT8 tensor cores (mma.sync u8)",
                                      "bit_identical_to_int64": bool(same8)},
             "backward_matmult_ms": {"p50": _pct(t_bwd, 0.5), "p99": _pct(t_bwd, 0.99)}, "max_abs_err": err,
-            "roofline": {"kernel": "cdiag_mac_kernel (+ rescale, whole call)", "bound": "alu", "achieved": round(achieved, 3),
-                         "peak": round(peak, 3), "unit": "T modmul-add/s", "frac": round(achieved / peak, 4),
-                         "peak_source": "derived: 64 IMAD/clk/SM x 152 SMs x 2070 MHz / 4 IMAD per 64-bit product"}}
+            "roofline": {"kernel": "cdiag_tc_mma_kernel (+ conversion and rescale, whole call)", "bound": "tensor", "achieved": round(achieved, 3),
+                         "peak": peak, "unit": "TFLOP/s bf16", "frac": round(achieved / peak, 4),
+                         "t_modmul_add_per_s": round(macs / (fwd_ms / 1e3) / 1e12, 3),
+                         "peak_source": peaks["source"]}}
 
 
 def run_batched(ctx, he, inputs, P, args, flush, world, dev):

@@ -96,7 +96,8 @@ void he_ctx_destroy(he_ctx *ctx);
  * context; forks and parent may be destroyed in any order.  he_keygen on one context may run
  * while the others work (the key table is guarded).  Waits for the parent's stream once. */
 int he_ctx_fork(he_ctx *parent, void *cuda_stream, he_ctx **out);
-/* Wait for every call issued on the context's stream. */
+/* Wait for every call issued on the context's stream.  HE_ETIMEOUT if a bounded wait of a kernel gave
+ * up (in any context of the family, at any time): results computed since are not to be used. */
 int he_synchronize(he_ctx *ctx);
 /* N of the ring and the prime count; any out pointer may be NULL. */
 int he_ctx_info(const he_ctx *ctx, int64_t *n, int32_t *n_q, int32_t *n_p);
@@ -271,7 +272,8 @@ int he_set_keyswitch_variant(he_ctx *ctx, int variant);
  * CTAs, the intermediate values in global memory; the inverse transform rows first; the ModUp of
  * he_rotate_many takes this form too).  The first matrix a
  * context encodes times the forms on its transform (synchronising the stream; not under stream
- * capture) and keeps the fastest for the context; he_ntt_form reports the choice (-1 before) and
+ * capture) and keeps the fastest for the context; he_ntt_form reports the choice (-1 before: form 2
+ * where it exists, else 0) and
  * ms[0..HE_NTT_FORMS-1] (may be NULL), he_set_ntt_form pins one (0 .. HE_NTT_FORMS-1, or -1 to
  * time again).  Results are the same in every form.  A fork starts with its parent's choice. */
 #define HE_NTT_FORMS 3
@@ -409,7 +411,9 @@ void he_server_free(he_server *s);
  * with the plaintext rotation done as the automorphism X -> X^(5^i) of w_k's plaintext (no
  * key switching: "eliminate all O4").  After decryption, he_cdiag_decode turns the K slot
  * vectors (device [K][N/2]) into Z = A W (device, m x K row-major), summing the n/m slot
- * groups when m < n (lazy rotate-and-sum, Sec. 4.3).  n_ct <= 1024 per call. */
+ * groups when m < n (lazy rotate-and-sum, Sec. 4.3).  n_ct <= 1024 per call.  With 8 and more columns
+ * the products run on the tensor cores, exactly (the same residues); he_cdiag_matmult returns
+ * HE_ETIMEOUT once a bounded wait of those kernels has given up (see he_synchronize). */
 typedef struct he_cdmat he_cdmat;
 int he_cdiag_encode_weights(he_ctx *ctx, const double *W, int64_t n, int64_t K, int level, he_cdmat **out);
 void he_cdmat_free(he_cdmat *W);
