@@ -886,6 +886,164 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(PENDING) : "memory");
 }
 
+// Accumulators of one coefficient's loop for primes q = 2^40 - delta, delta < 2^21: operands cut at 20 bits, products of the halves by
+// Karatsuba's method (three 32 x 32 -> 64-bit multiplies), each added to a 64-bit sum of its own, so
+// nothing carries between words.  A wide multiply-add takes the multiplier pipe four cycles per warp
+// and partition; a 64 x 64 -> 128-bit one is four of them and five carries, this one three.  The inner
+// sum (below 3 2^80) folds by 2^40 = delta twice to below 2^46 instead of a Montgomery reduction, and
+// the outer sums (products below 2^48) take 2^15 steps, more than any plan has, without one; finish
+// takes the Montgomery factors of key and plaintext out.
+struct MMAcc40 {
+    struct Sum {  // l + (p - l - h) 2^20 + h 2^40
+        uint64_t l, p, h;
+    };
+    Sum s0, s1, t0, t1, tc;
+    uint64_t q, qinv, mu;
+    uint32_t delta;
+    static __device__ __forceinline__ uint64_t wide(uint32_t a, uint32_t b, uint64_t c) { return (uint64_t)a * b + c; }
+    static __device__ __forceinline__ void cut(uint64_t x, uint32_t &lo, uint32_t &hi) {
+        lo = (uint32_t)x & 0xFFFFF;
+        hi = __funnelshift_r((uint32_t)x, (uint32_t)(x >> 32), 20);
+    }
+    static __device__ __forceinline__ void add(Sum &s, uint32_t a0, uint32_t a1, uint32_t as, uint32_t b0, uint32_t b1) {
+        s.l = wide(a0, b0, s.l);
+        s.h = wide(a1, b1, s.h);
+        s.p = wide(as, b0 + b1, s.p);
+    }
+    // below 2^46: l < 3 2^40, middle < 6 2^40, h < 3 2^40, so the first fold stays below 2^64
+    __device__ __forceinline__ uint64_t reduce(const Sum &s) const {
+        const uint64_t m = s.p - s.l - s.h;
+        uint64_t t = wide((uint32_t)s.h, delta, s.l) + (m << 20);
+        t += (uint64_t)((uint32_t)(s.h >> 32) * delta) << 32;
+        const uint32_t hi = (uint32_t)(t >> 32);
+        return wide(hi >> 8, delta, ((uint64_t)(hi & 0xFF) << 32) | (uint32_t)t);
+    }
+    __device__ __forceinline__ uint64_t total(const Sum &s) const {  // s 2^-64 mod q
+        return fold_wide((u128)s.l + ((u128)(s.p - s.l - s.h) << 20) + ((u128)s.h << 40), q, qinv, mu);
+    }
+    __device__ __forceinline__ void init(uint32_t delta_, uint64_t q_, uint64_t qinv_, uint64_t mu_) {
+        t0 = t1 = tc = s0 = s1 = Sum{0, 0, 0};
+        q = q_, qinv = qinv_, mu = mu_, delta = delta_;
+    }
+    __device__ __forceinline__ void begin() {
+        s0 = s1 = Sum{0, 0, 0};
+    }
+    __device__ __forceinline__ void digit(uint64_t d, uint64_t k0, uint64_t k1) {
+        uint32_t d0, d1, a, b;
+        cut(d, d0, d1);
+        const uint32_t ds = d0 + d1;
+        cut(k0, a, b);
+        add(s0, d0, d1, ds, a, b);
+        cut(k1, a, b);
+        add(s1, d0, d1, ds, a, b);
+    }
+    __device__ __forceinline__ void end(uint64_t p, uint64_t c, bool inq) {
+        uint32_t p0, p1, a, b;
+        cut(p, p0, p1);
+        cut(reduce(s0), a, b);
+        add(t0, a, b, a + b, p0, p1);
+        cut(reduce(s1), a, b);
+        add(t1, a, b, a + b, p0, p1);
+        if (inq) {
+            cut(c, a, b);
+            add(tc, a, b, a + b, p0, p1);
+        }
+    }
+    __device__ __forceinline__ void finish(uint64_t &o0, uint64_t &o1, uint64_t &oc) const {
+        o0 = redc(0, total(t0), q, qinv);  // the key's Montgomery factor besides the plaintext's
+        o1 = redc(0, total(t1), q, qinv);
+        oc = total(tc);
+    }
+};
+
+// The staged loop of mm_tile over one lane's rotation steps with 40-bit accumulators: the sums r0, r1
+// (key product times plaintext) and rc (c0 times plaintext).  The batch's persistent kernel, 95% of a
+// batch and bound by the multiplier pipe, takes it for its 40-bit limbs (two of four at the benchmark's
+// ring): 64 uneven jobs 7351 -> 6878 us, 235 instead of 299 cycles per unit in a micro-benchmark.  Single
+// products do not: beside the general path it left their two forms fewer registers (fused tables
+// 53 -> 63 us at 1024 x 256, 5000 x 300 with them 342 -> 487).
+constexpr uint64_t MM40_DELTA = 1 << 21;
+template <int ND, int VEC, int G, int S, bool GA>
+__device__ __forceinline__ void mm_sum40(const uint64_t *__restrict__ ct, const uint64_t *__restrict__ D, const uint64_t *__restrict__ pts,
+                                         const uint64_t *const *keys, const uint32_t *galois, int m_prime, int ext, int LK, int kl, bool inq, int u,
+                                         int k, int grp, const ModConst &m, int logn, uint64_t *pipe, uint64_t (&r0)[VEC], uint64_t (&r1)[VEC],
+                                         uint64_t (&rc)[VEC]) {
+    const int N = 1 << logn;
+    MMAcc40 acc[VEC];
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) acc[j].init((uint32_t)m.delta40, m.q, m.qinv, m.mu);
+    // stages, fields and gathers as in mm_tile
+    constexpr int F = 2 * ND + 1 + (GA ? ND + 1 : 0);
+    auto slot = [&](int st, int f) { return pipe + ((st * F + f) * MM_THREADS + (int)threadIdx.x) * VEC; };
+    uint32_t odd_bits = 0;
+    auto issue = [&](int t) {
+        const int i = 1 + grp + t * G;
+        if (i < m_prime) {
+            const int st = t % S;
+            const uint64_t *key = keys[i - 1] + (int64_t)kl * N + k;
+#pragma unroll
+            for (int f = 0; f < 2 * ND; ++f) cp_async<8 * VEC>(slot(st, f), key + (int64_t)f * LK * N);
+            cp_async<8 * VEC>(slot(st, 2 * ND), pts + ((int64_t)i * ext + u) * N + k);
+            if constexpr (GA) {
+                const uint32_t src = automorph_src(k, galois[i - 1], logn);
+                const uint32_t sa = VEC == 2 ? (src & ~1u) : src;
+                if constexpr (VEC == 2) odd_bits = (odd_bits & ~(1u << st)) | ((src & 1u) << st);
+#pragma unroll
+                for (int d = 0; d < ND; ++d) cp_async<8 * VEC>(slot(st, 2 * ND + 1 + d), D + ((int64_t)d * ext + u) * N + sa);
+                if (inq) cp_async<8 * VEC>(slot(st, 3 * ND + 1), ct + (int64_t)u * N + sa);
+            }
+        }
+        cp_async_commit();
+    };
+    uint64_t dv[ND][VEC], cv[VEC];
+    auto gather = [&](int t) {
+        const int i = 1 + grp + t * G;
+        if (i >= m_prime) return;
+        if constexpr (GA) {
+            const int st = t % S, odd = VEC == 2 ? (int)((odd_bits >> st) & 1u) : 0;
+#pragma unroll
+            for (int d = 0; d < ND; ++d)
+#pragma unroll
+                for (int j = 0; j < VEC; ++j) dv[d][j] = slot(st, 2 * ND + 1 + d)[j ^ odd];
+            if (inq)
+#pragma unroll
+                for (int j = 0; j < VEC; ++j) cv[j] = slot(st, 3 * ND + 1)[j ^ odd];
+        } else {
+            const uint32_t src = automorph_src(k, galois[i - 1], logn);
+#pragma unroll
+            for (int d = 0; d < ND; ++d) gatherv<VEC>(D + ((int64_t)d * ext + u) * N, src, dv[d]);
+            if (inq) gatherv<VEC>(ct + (int64_t)u * N, src, cv);
+        }
+    };
+#pragma unroll
+    for (int t = 0; t < S; ++t) issue(t);
+    if constexpr (!GA) gather(0);
+    for (int t = 0; 1 + grp + t * G < m_prime; ++t) {
+        cp_async_wait<S - 1>();
+        const int st = t % S;
+        if constexpr (GA) gather(t);
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) acc[j].begin();
+#pragma unroll
+        for (int d = 0; d < ND; ++d)
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) acc[j].digit(dv[d][j], slot(st, 2 * d)[j], slot(st, 2 * d + 1)[j]);
+        uint64_t pmc[VEC], c0v[VEC];
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) {
+            pmc[j] = slot(st, 2 * ND)[j];
+            c0v[j] = cv[j];
+        }
+        issue(t + S);
+        if constexpr (!GA) gather(t + 1);
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) acc[j].end(pmc[j], c0v[j], inq);
+    }
+    cp_async_wait<0>();
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) acc[j].finish(r0[j], r1[j], rc[j]);
+}
+
 // One block: `lanes` (<= MM_THREADS / G) lanes of VEC consecutive coefficients each, thread t
 // serving lane t % lanes in rotation group t / lanes; the calling thread's lane starts at
 // coefficient k of extended limb u (k >= N: no lane).  Every thread of the block calls it (it
@@ -942,7 +1100,13 @@ __device__ __forceinline__ void mm_tile(const uint64_t *__restrict__ ct, const u
     uint64_t r0[VEC], r1[VEC], rc[VEC];
 #pragma unroll
     for (int j = 0; j < VEC; ++j) r0[j] = r1[j] = rc[j] = 0;
-    if (k < N) {
+    bool small = false;  // a 40-bit prime's limb, in the batch
+    if constexpr (!KH && NDIG > 0 && S > 0) {
+        small = mc[p].delta40 != 0 && mc[p].delta40 < MM40_DELTA;
+        if (small && k < N)
+            mm_sum40<NDIG, VEC, G, S, GA>(ct, D, pts, keys, galois, m_prime, ext, LK, kl, inq, u, k, grp, mc[p], logn, pipe, r0, r1, rc);
+    }
+    if (k < N && !small) {
         u128 t0[VEC], t1[VEC], tc[VEC];
 #pragma unroll
         for (int j = 0; j < VEC; ++j) t0[j] = t1[j] = tc[j] = 0;
