@@ -254,7 +254,7 @@ int he_matmult_plain_cipher_noalloc(he_ctx *ctx, const he_plan *plan, const he_p
  * runs its transforms as one CTA per limb-poly with the usual thread count (variant 0), with
  * 512 threads and at most 64 registers (variant 1), or in two phases of small CTAs per transform
  * (variant 2, log N = 12..14: the NTT form 2 split into rows and columns, see he_ntt_form).  The
- * first such call on a context times them on its first 32 rotations (synchronising the stream; not
+ * first such call on a context times them on its first 64 rotations (synchronising the stream; not
  * under stream capture) and keeps the fastest: variant (-1 before) and ms[0..HE_KS_VARIANTS-1]
  * (may be NULL) report the choice and the timings.  Every variant gives the same residues. */
 #define HE_KS_VARIANTS 3

@@ -480,8 +480,9 @@ void launch_keyswitch_many(he_ctx *ctx, const RotJob *jobs, int count, int level
         if (pe2) cudaEventRecord(pe2[1], st);
     };
     // the first launch of at least 32 rotations on a context chooses the transform variant by timing
-    // each on its first 32 (the launches overwrite their outputs with the same values, so
-    // repeating them changes nothing); not under stream capture, where the usual thread count is taken
+    // each on its first 64 (on 32, the two phases were taken for 59 rotations at N = 2^12: 72 us for 66;
+    // on a whole chunk, the first transposition at N = 2^14 took longer than it need).  The launches
+    // overwrite their outputs with the same values, so repeating them changes nothing.  Not under stream capture, where the usual thread count is taken
     if (ctx->ks_variant < 0 && cmax >= 32 && !use_cluster(logn, cmax * 2 * (level + 1))) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         cudaStreamIsCapturing(st, &cs);
@@ -492,7 +493,7 @@ void launch_keyswitch_many(he_ctx *ctx, const RotJob *jobs, int count, int level
                 float ms = 1e30f;
                 for (int rep = 0; rep < 3; ++rep) {
                     cudaEventRecord(e0, st);
-                    issue(0, v, 32);
+                    issue(0, v, 64);
                     cudaEventRecord(e1, st);
                     if (cudaEventSynchronize(e1) != cudaSuccess) break;
                     float t = 0.0f;
