@@ -55,21 +55,14 @@ namespace cg = cooperative_groups;
 
 namespace {
 
-constexpr int TC_ROWS = 64;                 // rows of a tile: 2 components x 32 coefficients
-constexpr int TC_KC = 64;                   // indices s per chunk (128 bytes of bfloat16: one swizzle row)
-constexpr int TC_DIAGS = 256;               // diagonals per pass: 255^2 256 < 2^24
-constexpr int TC_A_BYTES = TC_COLS * TC_KC * 2, TC_B_BYTES = TC_ROWS * TC_KC * 2, TC_STAGE_BYTES = TC_A_BYTES + TC_B_BYTES;
-constexpr int TC_CL = 2;                    // CTAs of a cluster: consecutive tiles that share the weights' window
+constexpr int TC_STAGE_BYTES = TC_A_BYTES + TC_B_BYTES;
 constexpr int TC_STAGES = 6, TC_SLOTS = 8;  // ring of operand stages; accumulators in tensor memory, TC_ROWS columns each
 constexpr int TC_FOLD_WARPS = 16, TC_THREADS = 32 * (2 + TC_FOLD_WARPS);
 constexpr int TC_TR_WORDS = 32 * 17;        // a fold warp's transposition: 32 columns by 16 rows, one pad word
 constexpr int TC_SMEM = TC_STAGES * TC_STAGE_BYTES + TC_FOLD_WARPS * TC_TR_WORDS * 8 + 8 * (2 * TC_STAGES + 2 * TC_SLOTS) + 16;
 constexpr int TC_TMEM_COLS = TC_SLOTS * TC_ROWS;
-constexpr int64_t TC_SLICE_BYTES = 96ll << 20;  // of the 126 MB L2
 constexpr int TC_RES_THREADS = 512;         // residues kernel: thread (row, octet of a chunk)
 constexpr unsigned TC_WAIT_LIMIT = 1u << 21;  // polls of a barrier (each suspended for a while by the hardware) before giving up
-// odd, pairwise coprime, below 512
-constexpr int TC_MODULI[TC_MAX_MOD] = {511, 509, 507, 503, 499, 493, 491, 487, 485, 479, 473, 467, 463, 461, 457};
 
 // per limb: the moduli count and the reconstruction constants
 struct TcLimb {
@@ -518,18 +511,6 @@ void digits20(int32_t (&d)[3], uint64_t v, uint64_t q, int nd) {
 
 }  // namespace
 
-// moduli count for the prime q: prod p_i > 2.01 TC_DIAGS q (q / 2); 0 where the three 20-bit digits
-// of the reconstruction do not hold a residue
-static int tc_moduli(uint64_t q) {
-    if (q >> 60) return 0;
-    long double need = 2.01L * TC_DIAGS * (long double)q * ((long double)q / 2), have = 1;
-    for (int m = 0; m < TC_MAX_MOD; ++m) {
-        have *= TC_MODULI[m];
-        if (have > need) return m + 1;
-    }
-    return 0;
-}
-
 bool cdiag_tc_supported(const he_ctx *ctx, int level, int64_t n) {
     if (ctx->log_n < 12 || ctx->log_n > 14 || n < 8) return false;
     for (int u = 0; u <= level; ++u)
@@ -593,45 +574,34 @@ void cdiag_tc_free(CdiagTc *tc) {
     tc->wt = nullptr;
 }
 
-// chunks of the longest window of cnt diagonals: its start is rounded down to a whole chunk from the
-// first block of a cluster's tiles, a multiple of the span (at most 64) of their blocks: 64 - span,
-// span - 1 and the diagonals
-static int tc_chunks(int cnt) { return (TC_KC - 1 + cnt + TC_KC - 1) / TC_KC; }
-static int64_t tc_tile_bytes(const he_ctx *ctx, int cnt, int level) {
+static int tc_max_moduli(const he_ctx *ctx, int level) {
     int mods = 0;
     for (int u = 0; u <= level; ++u) mods = std::max(mods, tc_moduli(ctx->primes[u]));
-    return (int64_t)mods * tc_chunks(cnt) * TC_B_BYTES;
-}
-// tiles of a slice: a whole number per SM (an even count of SMs), their operands at most TC_SLICE_BYTES (one tile per SM at
-// least), so that they are still in L2 when the product kernel reads them
-static int tc_slice(const he_ctx *ctx, int64_t tile_bytes) {
-    const int sms = ctx->sms / TC_CL * TC_CL;
-    return sms * (int)std::max<int64_t>(1, TC_SLICE_BYTES / (tile_bytes * sms));
+    return mods;
 }
 size_t cdiag_tc_words(const he_ctx *ctx, int n_ct, int level) {
-    const int64_t b = tc_tile_bytes(ctx, std::min(n_ct, TC_DIAGS), level);
-    return (size_t)std::min<int64_t>(tc_slice(ctx, b), (level + 1) * (ctx->n / 32)) * b / 8;
+    return (size_t)tc_scratch_bytes(ctx->sms, (level + 1) * (ctx->n / 32), tc_max_moduli(ctx, level), n_ct) / 8;
 }
 
 void cdiag_tc_mac(he_ctx *ctx, const CdiagTc *tc, const he_ct *cts, int n_ct, int level, int64_t K, uint64_t *pre, uint64_t *scratch) {
-    const int nl = level + 1, col_blocks = (int)((K + TC_COLS - 1) / TC_COLS), all = nl * (ctx->n / 32);
+    const int nl = level + 1, col_blocks = (int)((K + TC_COLS - 1) / TC_COLS), all = nl * (ctx->n / 32), mods = tc_max_moduli(ctx, level);
     unsigned char *X = reinterpret_cast<unsigned char *>(scratch);
     const TcLimb *limbs = static_cast<const TcLimb *>(ctx->d_tc);
     for (int i0 = 0; i0 < n_ct; i0 += TC_DIAGS) {
         TcGeom g{};
-        g.cnt = std::min(TC_DIAGS, n_ct - i0);
+        const TcPass pass = tc_pass(ctx->sms, mods, n_ct, i0);
+        g.cnt = pass.cnt;
         g.i0 = i0;
         g.nl = nl;
         g.K = (int)K;
         g.logn = ctx->log_n;
         g.lg_n = tc->lg_n;
         g.accumulate = i0 > 0;
-        g.chunks = tc_chunks(g.cnt);
-        g.tile_bytes = tc_tile_bytes(ctx, g.cnt, level);
+        g.chunks = pass.chunks;
+        g.tile_bytes = pass.tile_bytes;
         for (int i = 0; i < g.cnt; ++i) g.ct[i] = cts[i0 + i].data;
-        const int slice = tc_slice(ctx, g.tile_bytes);
-        for (g.first = 0; g.first < all; g.first += slice) {
-            g.tiles = std::min(slice, all - g.first);
+        for (g.first = 0; g.first < all; g.first += pass.slice) {
+            g.tiles = std::min(pass.slice, all - g.first);
             ctx->launches += 2;
             launch_k(cdiag_tc_residues_kernel, dim3((unsigned)g.tiles, (unsigned)g.chunks), TC_RES_THREADS, 0, ctx->stream, g, limbs, X);
             launch_cluster_n(cdiag_tc_mma_kernel, std::min(ctx->sms / TC_CL * TC_CL, g.tiles * col_blocks), TC_THREADS, TC_SMEM, ctx->stream, TC_CL, g,

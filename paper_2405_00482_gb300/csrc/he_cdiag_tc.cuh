@@ -2,10 +2,8 @@
 #pragma once
 #include <stdint.h>
 
+#include "he_cdiag_tc_plan.h"
 #include "he_internal.cuh"
-
-#define TC_COLS 128     // weight columns per tile (the instruction's M)
-#define TC_MAX_MOD 15
 
 // the weights of a he_cdmat as residues for the tensor cores
 struct CdiagTc {
@@ -19,6 +17,6 @@ bool cdiag_tc_supported(const he_ctx *ctx, int level, int64_t n);
 // tc from the encoded columns (device, [K][level+1][N], NTT form, canonical)
 int cdiag_tc_prepare(he_ctx *ctx, CdiagTc *tc, int64_t n, int64_t K, int level, const uint64_t *cols);
 void cdiag_tc_free(CdiagTc *tc);
-// pre [K][2][level+1][N] = the products' sums over the n_ct ciphertexts
+// pre [K][2][level+1][N] = the products' sums over the n_ct ciphertexts; scratch: cdiag_tc_words
 void cdiag_tc_mac(he_ctx *ctx, const CdiagTc *tc, const he_ct *cts, int n_ct, int level, int64_t K, uint64_t *pre, uint64_t *scratch);
-size_t cdiag_tc_words(const he_ctx *ctx, int n_ct, int level);  // its scratch
+size_t cdiag_tc_words(const he_ctx *ctx, int n_ct, int level);

@@ -1,0 +1,65 @@
+// he_cdiag_tc_plan.h -- sizes of the tensor-core ciphertext-diagonal product (he_cdiag_tc.cu): tiles,
+// passes over the diagonals, slices of tiles and the scratch that holds a slice's operands.  Plain C++,
+// without CUDA, so that a host test can walk every pass.
+#pragma once
+#include <stdint.h>
+
+#include <algorithm>
+
+constexpr int TC_COLS = 128;                // weight columns per tile (the instruction's M)
+constexpr int TC_ROWS = 64;                 // rows of a tile: 2 components x 32 coefficients
+constexpr int TC_KC = 64;                   // indices s per chunk (128 bytes of bfloat16: one swizzle row)
+constexpr int TC_DIAGS = 256;               // diagonals per pass: 255^2 256 < 2^24
+constexpr int TC_CL = 2;                    // CTAs of a cluster: consecutive tiles that share the weights' window
+constexpr int TC_A_BYTES = TC_COLS * TC_KC * 2, TC_B_BYTES = TC_ROWS * TC_KC * 2;
+constexpr int64_t TC_SLICE_BYTES = 96ll << 20;  // of the 126 MB L2
+constexpr int TC_MAX_MOD = 15;
+// odd, pairwise coprime, below 512
+constexpr int TC_MODULI[TC_MAX_MOD] = {511, 509, 507, 503, 499, 493, 491, 487, 485, 479, 473, 467, 463, 461, 457};
+
+// moduli count for the prime q: prod p_i > 2.01 TC_DIAGS q (q / 2); 0 where the three 20-bit digits
+// of the reconstruction do not hold a residue
+inline int tc_moduli(uint64_t q) {
+    if (q >> 60) return 0;
+    long double need = 2.01L * TC_DIAGS * (long double)q * ((long double)q / 2), have = 1;
+    for (int m = 0; m < TC_MAX_MOD; ++m) {
+        have *= TC_MODULI[m];
+        if (have > need) return m + 1;
+    }
+    return 0;
+}
+
+// chunks of the longest window of cnt diagonals: its start is rounded down to a whole chunk from the
+// first block of a cluster's tiles, a multiple of the span (at most 64) of their blocks: 64 - span,
+// span - 1 and the diagonals
+inline int tc_chunks(int cnt) { return (TC_KC - 1 + cnt + TC_KC - 1) / TC_KC; }
+
+// the pass over the diagonals i0 .. i0 + cnt of n_ct, on operands of up to `mods` moduli
+struct TcPass {
+    int cnt, chunks;
+    int64_t tile_bytes;  // operand blocks of a tile: [modulus][chunk][64 rows x 128 bytes]
+    int slice;           // tiles of a slice: a whole number per SM (an even count of SMs), their operands at
+                         // most TC_SLICE_BYTES (one tile per SM at least), so that they are still in L2
+                         // when the product kernel reads them
+};
+inline TcPass tc_pass(int sms, int mods, int n_ct, int i0) {
+    TcPass p;
+    p.cnt = std::min(TC_DIAGS, n_ct - i0);
+    p.chunks = tc_chunks(p.cnt);
+    p.tile_bytes = (int64_t)mods * p.chunks * TC_B_BYTES;
+    const int even = sms / TC_CL * TC_CL;
+    p.slice = even * (int)std::max<int64_t>(1, TC_SLICE_BYTES / (p.tile_bytes * even));
+    return p;
+}
+
+// operand scratch of a product of n_ct diagonals over `tiles` tiles: the largest slice of any pass.  A
+// short last pass has smaller tiles but more of them in a slice, and can need more than a full one (10
+// moduli, 152 SMs: 62 MB for 256 diagonals, 100 MB for the 44 left of 300).
+inline int64_t tc_scratch_bytes(int sms, int tiles, int mods, int n_ct) {
+    int64_t bytes = 0;
+    for (int i0 = 0; i0 < n_ct; i0 += TC_DIAGS) {
+        const TcPass p = tc_pass(sms, mods, n_ct, i0);
+        bytes = std::max(bytes, std::min(p.slice, tiles) * p.tile_bytes);
+    }
+    return bytes;
+}

@@ -1,0 +1,53 @@
+"""The operand scratch of the tensor-core ciphertext-diagonal product holds every slice of every pass,
+for all diagonal counts (no GPU: the sizes' header compiled by the host compiler)."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2405_00482_gb300", "csrc")
+SRC = """
+#include "he_cdiag_tc_plan.h"
+// the loops of cdiag_tc_mac: bytes written by the largest slice of any pass
+extern "C" int64_t used(int sms, int tiles, int mods, int n_ct) {
+    int64_t most = 0;
+    for (int i0 = 0; i0 < n_ct; i0 += TC_DIAGS) {
+        const TcPass p = tc_pass(sms, mods, n_ct, i0);
+        for (int first = 0; first < tiles; first += p.slice)
+            most = std::max(most, std::min(p.slice, tiles - first) * p.tile_bytes);
+    }
+    return most;
+}
+extern "C" int64_t scratch(int sms, int tiles, int mods, int n_ct) { return tc_scratch_bytes(sms, tiles, mods, n_ct); }
+extern "C" int moduli(uint64_t q) { return tc_moduli(q); }
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("plan")
+    (d / "plan.cpp").write_text(SRC)
+    so = str(d / "plan.bin")
+    subprocess.run(["g++", "-std=c++20", "-O1", "-shared", "-fPIC", "-I", CSRC, str(d / "plan.cpp"), "-o", so], check=True)
+    lib = ctypes.CDLL(so)
+    for f in (lib.used, lib.scratch):
+        f.restype, f.argtypes = ctypes.c_int64, [ctypes.c_int] * 4
+    lib.moduli.argtypes = [ctypes.c_uint64]
+    return lib
+
+
+@pytest.mark.parametrize("tiles", [128, 256, 512, 768, 3584])
+@pytest.mark.parametrize("sms", [132, 148, 152])
+def test_scratch_holds_every_pass(lib, sms, tiles):
+    for mods in range(1, 16):
+        for n_ct in range(1, 1025):
+            assert lib.used(sms, tiles, mods, n_ct) <= lib.scratch(sms, tiles, mods, n_ct), (mods, n_ct)
+
+
+def test_a_short_last_pass_can_need_more_than_a_full_one(lib):
+    """The N = 2^12 ring's and an all-40-bit chain's moduli, the diagonal counts that outgrew a scratch of the first pass's size."""
+    mods = lib.moduli((1 << 40) - 87)
+    assert mods == 10
+    assert lib.scratch(152, 512, mods, 256) < lib.scratch(152, 512, mods, 300) == lib.used(152, 512, mods, 300)
+    assert lib.scratch(152, 256, mods, 256) < lib.scratch(152, 256, mods, 449) == lib.used(152, 256, mods, 449)
