@@ -1212,8 +1212,10 @@ int he_matmult_plain_cipher(he_ctx *ctx, const he_plan *plan, const he_ptmat *pm
             finish(++r, acc + wa, nullptr);
             continue;
         }
-        // one diagonal, one column block: the product and its rescale in one launch
-        if (!rot && C == 1 && launch_product_rescale(ctx, ins[0].data, pm->data + (size_t)r * pm->ext * N, level, outs[r].data)) continue;
+        // one diagonal, one column block: the product and its rescale in one launch, whose clusters write
+        // outs[r] while others still read ins[0]; an output in its input's buffer goes through scratch
+        const bool apart = outs[r].data + 2 * (size_t)level * N <= ins[0].data || ins[0].data + 2 * nl * N <= outs[r].data;
+        if (!rot && C == 1 && apart && launch_product_rescale(ctx, ins[0].data, pm->data + (size_t)r * pm->ext * N, level, outs[r].data)) continue;
         for (size_t c = 0; c < C; ++c)
             launch_matmult_loop(ctx, pm, r, (int)c, ins[c].data, rot ? D + c * mu.ndig * ext * N : nullptr, acc, cacc, c > 0);
         if (rot)
