@@ -31,27 +31,25 @@
 // one CTA doing both in turn, took 1.55 ms where the two kernels take 1.07: the registers of the
 // reconstruction left none for the conversion, whose instructions it then waited for.)
 //
-// The product kernel is specialised by warp: one thread copies (bulk copies; a cluster of two CTAs
-// shares the weights' window, each CTA multicasting half of every block) through a ring of stages, one
-// warp issues the tcgen05.mma (M 128, N 64, K 16), and 16 warps fold each modulus' sums from tensor
-// memory (8 slots of 64 columns) into the reconstruction's registers, all three running ahead of each
-// other by their rings.  The results go through shared memory so that half a warp stores 16 rows of
-// one column (stored from the registers, one column per lane, they took 8.5 of a slice's 40 us).
+// The product kernel is specialised by warp: one thread copies the weights' and the tile's blocks (bulk
+// copies) through a ring of stages, one warp issues the tcgen05.mma (M 128, N 64, K 16), and 16 warps
+// fold each modulus' sums from tensor memory (8 slots of 64 columns) into the reconstruction's
+// registers, all three running ahead of each other by their rings.  Every CTA copies all of the weights'
+// blocks for itself: the copies are not what it waits for (halves multicast within a pair of CTAs took
+// the same time, 1.50 against 1.49 ms for the whole call), and a multicast load has no place in a library
+// that also runs on several GPUs.  The results go through shared memory so that half a warp stores 16
+// rows of one column (stored from the registers, one column per lane, they took 8.5 of a slice's 40 us).
 //
 // 4096 x 256 activations (256 diagonals) by 128 columns at N = 2^14, 7 limbs: 7.5 G modular
 // multiply-adds in 0.44 ms (residues: float and integer issue, 65% active) and 0.63 ms (products:
 // the issue of short tensor instructions, about 100 cycles each, and the start and end of each slice),
 // against 6.26 ms for the 64-bit integer form (cdiag_mac_kernel), which the multiplier pipe bounds.
 
-#include <cooperative_groups.h>
-
 #include <algorithm>
 #include <vector>
 
 #include "he_cdiag_tc.cuh"
 #include "he_internal.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace {
 
@@ -130,12 +128,7 @@ __device__ __forceinline__ bool elect_one() {
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
     return p != 0;
 }
-// arrives on bar of every CTA of the cluster once the products issued so far are complete
-__device__ __forceinline__ void umma_commit_cluster(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-                 "h"((uint16_t)((1 << TC_CL) - 1))
-                 : "memory");
-}
+// arrives on bar once the products issued so far are complete
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
@@ -221,10 +214,9 @@ __device__ __forceinline__ TcTile tc_tile_of(const TcGeom &g, int tile) {
     const int in_orbit = rt & ((1 << lg_orbit) - 1);
     t.j0 = (in_orbit >> lg_sub) << lg_t;
     t.p0 = (in_orbit & ((1 << lg_sub) - 1)) << t.lg_pt;
-    // the window starts at a whole chunk of the weights, for all tiles of a cluster: at or before the
-    // first block of the first tile; it holds the diagonals of the last tile's last block
-    const int cl0 = in_orbit & ~(TC_CL - 1), j_first = ((cl0 >> lg_sub) << lg_t) + g.i0,
-              j_last = (((cl0 + TC_CL - 1) >> lg_sub) << lg_t) + (1 << lg_t) - 1 + g.i0;
+    // the window starts at a whole chunk of the weights, at or before the tile's first block, and holds
+    // the diagonals of its last block
+    const int j_first = t.j0 + g.i0, j_last = j_first + (1 << lg_t) - 1;
     t.s0 = j_first & ~(TC_KC - 1);
     t.step0 = (j_first - t.s0) >> 4;
     t.step1 = (j_last - t.s0 + g.cnt + 15) >> 4;
@@ -348,8 +340,8 @@ __device__ __forceinline__ bool tc_fold(const TcGeom &g, const TcTile &t, int kb
     return ok;
 }
 
-// Units: the slice's tiles by blocks of 128 columns; the CTAs of a cluster take consecutive tiles
-// (same limb, orbit and window) and each copies its share of the weights' rows to all of them.
+// Units: the slice's tiles by blocks of 128 columns; neighbouring CTAs take consecutive tiles (same limb,
+// orbit and nearly the same window), so the weights' blocks that each copies for itself come from L2.
 __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __grid_constant__ TcGeom g, const __grid_constant__ CdiagTc tc,
                                                                      const TcLimb *__restrict__ limbs, const unsigned char *__restrict__ X, uint64_t *pre,
                                                                      const ModConst *__restrict__ mc, unsigned int *err) {
@@ -363,20 +355,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
     if (threadIdx.x == 0) {
         for (int i = 0; i < TC_STAGES; ++i) {
             mbar_init(full + 8 * i, 1);
-            mbar_init(empty + 8 * i, TC_CL);  // the products of every CTA: the weights are multicast
+            mbar_init(empty + 8 * i, 1);
         }
         for (int i = 0; i < TC_SLOTS; ++i) {
             mbar_init(acc_full + 8 * i, 1);
             mbar_init(acc_empty + 8 * i, TC_FOLD_WARPS);
         }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");  // for the copies' and products' arrivals
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tmem_slot), "n"(TC_TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    cg::this_cluster().sync();  // the peers' barriers exist before anything arrives on them
+    __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(bars + 2 * TC_STAGES + 2 * TC_SLOTS);
     HE_GRID_WAIT();
@@ -386,12 +378,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
         if (lane == 0) {  // copies
             asm volatile("fence.proxy.async;" ::: "memory");  // the residues were written through the generic proxy
             uint32_t it = 0;
-            const int rank = (int)cg::this_cluster().block_rank();
             for (int unit = blockIdx.x; unit < units && ok; unit += gridDim.x) {
                 const int lt = unit % g.tiles, kb = unit / g.tiles;
                 const TcTile t = tc_tile_of(g, g.first + lt);
                 const int n_mod = limbs[t.u].n_mod, wchunks = max(1, (1 << g.lg_n) / TC_KC);
-                const unsigned char *w = tc.wt + tc.block[t.u] * TC_A_BYTES + rank * (TC_A_BYTES / TC_CL);
+                const unsigned char *w = tc.wt + tc.block[t.u] * TC_A_BYTES;
                 const unsigned char *x = X + lt * g.tile_bytes;
                 for (int m = 0; m < n_mod && ok; ++m)
                     for (int c = t.step0 / 4; c * 4 < t.step1 && ok; ++c, ++it) {
@@ -400,13 +391,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
                         if (!ok) break;
                         const uint32_t bar = full + 8 * st, A = full_stage + st * TC_STAGE_BYTES;
                         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(TC_STAGE_BYTES) : "memory");
-                        // this CTA's share of the weights' block, to every CTA of the cluster
                         const int64_t b = ((int64_t)(2 * m + t.orbit) * col_blocks + kb) * wchunks + ((t.s0 / TC_KC + c) & (wchunks - 1));
-                        asm volatile(
-                            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1], %2, [%3], %4;" ::"r"(
-                                A + rank * (TC_A_BYTES / TC_CL)),
-                            "l"(w + b * TC_A_BYTES), "r"(TC_A_BYTES / TC_CL), "r"(bar), "h"((uint16_t)((1 << TC_CL) - 1))
-                            : "memory");
+                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(A),
+                                     "l"(w + b * TC_A_BYTES), "r"(TC_A_BYTES), "r"(bar)
+                                     : "memory");
                         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(A + TC_A_BYTES),
                                      "l"(x + ((int64_t)m * g.chunks + c) * TC_B_BYTES), "r"(TC_B_BYTES), "r"(bar)
                                      : "memory");
@@ -434,7 +422,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
                             if (c * 4 + k >= t.step0 && c * 4 + k < t.step1) umma(d, da + 2 * k, db + 2 * k, c * 4 + k > t.step0);
-                        umma_commit_cluster(empty + 8 * st);
+                        umma_commit(empty + 8 * st);
                         if ((c + 1) * 4 >= t.step1) umma_commit(acc_full + 8 * slot);
                     }
                     __syncwarp();
@@ -452,11 +440,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
         }
     }
     if (!ok) atomicExch(err, 1u);
-    // every copy and product was consumed (or a wait gave up after seconds): the tensor memory is
-    // free, and no peer copies into this CTA or arrives on its barriers any more
+    // every copy and product was consumed (or a wait gave up after seconds): the tensor memory is free
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncwarp();
-    cg::this_cluster().sync();
+    __syncthreads();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(TC_TMEM_COLS) : "memory");
 }
 
@@ -604,8 +591,8 @@ void cdiag_tc_mac(he_ctx *ctx, const CdiagTc *tc, const he_ct *cts, int n_ct, in
             g.tiles = std::min(pass.slice, all - g.first);
             ctx->launches += 2;
             launch_k(cdiag_tc_residues_kernel, dim3((unsigned)g.tiles, (unsigned)g.chunks), TC_RES_THREADS, 0, ctx->stream, g, limbs, X);
-            launch_cluster_n(cdiag_tc_mma_kernel, std::min(ctx->sms / TC_CL * TC_CL, g.tiles * col_blocks), TC_THREADS, TC_SMEM, ctx->stream, TC_CL, g,
-                             *tc, limbs, (const unsigned char *)X, pre, (const ModConst *)ctx->d_mc, ctx->sh->dev_err);
+            launch_k(cdiag_tc_mma_kernel, std::min(ctx->sms, g.tiles * col_blocks), TC_THREADS, TC_SMEM, ctx->stream, g, *tc, limbs,
+                     (const unsigned char *)X, pre, (const ModConst *)ctx->d_mc, ctx->sh->dev_err);
         }
     }
 }

@@ -10,7 +10,6 @@ constexpr int TC_COLS = 128;                // weight columns per tile (the inst
 constexpr int TC_ROWS = 64;                 // rows of a tile: 2 components x 32 coefficients
 constexpr int TC_KC = 64;                   // indices s per chunk (128 bytes of bfloat16: one swizzle row)
 constexpr int TC_DIAGS = 256;               // diagonals per pass: 255^2 256 < 2^24
-constexpr int TC_CL = 2;                    // CTAs of a cluster: consecutive tiles that share the weights' window
 constexpr int TC_A_BYTES = TC_COLS * TC_KC * 2, TC_B_BYTES = TC_ROWS * TC_KC * 2;
 constexpr int64_t TC_SLICE_BYTES = 96ll << 20;  // of the 126 MB L2
 constexpr int TC_MAX_MOD = 15;
@@ -30,25 +29,24 @@ inline int tc_moduli(uint64_t q) {
 }
 
 // chunks of the longest window of cnt diagonals: its start is rounded down to a whole chunk from the
-// first block of a cluster's tiles, a multiple of the span (at most 64) of their blocks: 64 - span,
-// span - 1 and the diagonals
+// tile's first block, a multiple of the span (at most 32) of its blocks: 64 - span, span - 1 and the
+// diagonals
 inline int tc_chunks(int cnt) { return (TC_KC - 1 + cnt + TC_KC - 1) / TC_KC; }
 
 // the pass over the diagonals i0 .. i0 + cnt of n_ct, on operands of up to `mods` moduli
 struct TcPass {
     int cnt, chunks;
     int64_t tile_bytes;  // operand blocks of a tile: [modulus][chunk][64 rows x 128 bytes]
-    int slice;           // tiles of a slice: a whole number per SM (an even count of SMs), their operands at
-                         // most TC_SLICE_BYTES (one tile per SM at least), so that they are still in L2
-                         // when the product kernel reads them
+    int slice;           // tiles of a slice: a whole number per SM, their operands at most TC_SLICE_BYTES
+                         // (one tile per SM at least), so that they are still in L2 when the product kernel
+                         // reads them
 };
 inline TcPass tc_pass(int sms, int mods, int n_ct, int i0) {
     TcPass p;
     p.cnt = std::min(TC_DIAGS, n_ct - i0);
     p.chunks = tc_chunks(p.cnt);
     p.tile_bytes = (int64_t)mods * p.chunks * TC_B_BYTES;
-    const int even = sms / TC_CL * TC_CL;
-    p.slice = even * (int)std::max<int64_t>(1, TC_SLICE_BYTES / (p.tile_bytes * even));
+    p.slice = sms * (int)std::max<int64_t>(1, TC_SLICE_BYTES / (p.tile_bytes * sms));
     return p;
 }
 
