@@ -35,9 +35,8 @@
 // copies) through a ring of stages, one warp issues the tcgen05.mma (M 128, N 64, K 16), and 16 warps
 // fold each modulus' sums from tensor memory (8 slots of 64 columns) into the reconstruction's
 // registers, all three running ahead of each other by their rings.  Every CTA copies all of the weights'
-// blocks for itself: the copies are not what it waits for (halves multicast within a pair of CTAs took
-// the same time, 1.50 against 1.49 ms for the whole call), and a multicast load has no place in a library
-// that also runs on several GPUs.  The results go through shared memory so that half a warp stores 16
+// blocks for itself: the copies are not what it waits for (halves shared within a pair of CTAs took the
+// same time, 1.50 against 1.49 ms for the whole call).  The results go through shared memory so that half a warp stores 16
 // rows of one column (stored from the registers, one column per lane, they took 8.5 of a slice's 40 us).
 //
 // 4096 x 256 activations (256 diagonals) by 128 columns at N = 2^14, 7 limbs: 7.5 G modular
@@ -349,7 +348,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
     extern __shared__ __align__(1024) unsigned char smem_tc[];  // the swizzle repeats every 1024 bytes
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem_tc + TC_STAGES * TC_STAGE_BYTES) + TC_FOLD_WARPS * TC_TR_WORDS;
     const uint32_t full = smem_u32(bars), empty = full + 8 * TC_STAGES, acc_full = empty + 8 * TC_STAGES, acc_empty = acc_full + 8 * TC_SLOTS,
-                   tmem_slot = acc_empty + 8 * TC_SLOTS;
+                   tmem_slot = acc_empty + 8 * TC_SLOTS, drained = tmem_slot + 8;
     const uint32_t full_stage = smem_u32(smem_tc);
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp-uniform
     if (threadIdx.x == 0) {
@@ -361,6 +360,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
             mbar_init(acc_full + 8 * i, 1);
             mbar_init(acc_empty + 8 * i, TC_FOLD_WARPS);
         }
+        mbar_init(drained, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");  // for the copies' and products' arrivals
     }
     if (warp == 0) {
@@ -400,6 +400,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
                                      : "memory");
                     }
             }
+            // no copy may land after this CTA: where a wait gave up, here or in the other warps, nobody else
+            // waits for the last ones (otherwise they are long complete)
+            for (uint32_t i = it < TC_STAGES ? 0 : it - TC_STAGES; i < it; ++i)
+                if (!mbar_wait(full + 8 * (i % TC_STAGES), (int)((i / TC_STAGES) & 1), true)) ok = false;
         }
     } else if (warp == 1) {
         // products: the whole warp walks the rings, one elected lane issues, so that descriptors and
@@ -429,6 +433,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
                 }
             }
         }
+        // likewise the products: none may write tensor memory that has been given back
+        if (elect_one()) umma_commit(drained);
+        __syncwarp();
+        if (!mbar_wait(drained, 0, true)) ok = false;
     } else {
         uint32_t slot_it = 0;
         uint64_t *tr = bars - (TC_FOLD_WARPS - (warp - 2)) * TC_TR_WORDS;
@@ -440,7 +448,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
         }
     }
     if (!ok) atomicExch(err, 1u);
-    // every copy and product was consumed (or a wait gave up after seconds): the tensor memory is free
+    // every copy and product is complete: the tensor memory is free
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncwarp();
     __syncthreads();
