@@ -96,9 +96,19 @@ void he_ctx_destroy(he_ctx *ctx);
  * context; forks and parent may be destroyed in any order.  he_keygen on one context may run
  * while the others work (the key table is guarded).  Waits for the parent's stream once. */
 int he_ctx_fork(he_ctx *parent, void *cuda_stream, he_ctx **out);
-/* Wait for every call issued on the context's stream.  HE_ETIMEOUT if a bounded wait of a kernel gave
- * up (in any context of the family, at any time): results computed since are not to be used. */
+/* Wait for every call issued on the context's stream.  HE_ETIMEOUT, once, if a bounded wait of a kernel
+ * gave up in any context of the family since this context's last he_synchronize: results of the
+ * tensor-core products (he_cdiag_matmult) computed since then are not to be used.  From the moment
+ * it is known and until he_synchronize has reported it, he_decrypt, he_matmult_decrypt,
+ * he_cdiag_decode, their host-memory forms, he_ct_export_host and he_cdiag_matmult on the tensor cores
+ * return HE_ETIMEOUT too.  Calls are asynchronous: one issued before the failing kernel has ended
+ * cannot know, so a program that reads such results in stream order alone calls he_synchronize (or
+ * one of those calls) once before it relies on them. */
 int he_synchronize(he_ctx *ctx);
+/* Polls of a barrier after which a kernel's wait gives up on this context: 0 (gives up at once, which
+ * tests a program's handling of HE_ETIMEOUT) .. 2^21, the default (seconds; a wait normally takes
+ * microseconds). */
+int he_set_wait_limit(he_ctx *ctx, int64_t polls);
 /* N of the ring and the prime count; any out pointer may be NULL. */
 int he_ctx_info(const he_ctx *ctx, int64_t *n, int32_t *n_q, int32_t *n_p);
 
@@ -412,8 +422,8 @@ void he_server_free(he_server *s);
  * key switching: "eliminate all O4").  After decryption, he_cdiag_decode turns the K slot
  * vectors (device [K][N/2]) into Z = A W (device, m x K row-major), summing the n/m slot
  * groups when m < n (lazy rotate-and-sum, Sec. 4.3).  n_ct <= 1024 per call.  With 8 and more columns
- * the products run on the tensor cores, exactly (the same residues); he_cdiag_matmult returns
- * HE_ETIMEOUT once a bounded wait of those kernels has given up (see he_synchronize). */
+ * the products run on the tensor cores, exactly (the same residues), in kernels with bounded waits
+ * (HE_ETIMEOUT: see he_synchronize). */
 typedef struct he_cdmat he_cdmat;
 int he_cdiag_encode_weights(he_ctx *ctx, const double *W, int64_t n, int64_t K, int level, he_cdmat **out);
 void he_cdmat_free(he_cdmat *W);

@@ -415,11 +415,11 @@ int he_ctx_create(const he_params *p, uint64_t seed, void *stream, he_ctx **out)
         }
         ctx->moddown.push_back(md);
     }
-    if (cudaHostAlloc(&ctx->sh->dev_err, sizeof(unsigned int), cudaHostAllocMapped) != cudaSuccess) {
+    if (cudaHostAlloc(&ctx->sh->gave_up, sizeof(unsigned int), cudaHostAllocMapped) != cudaSuccess) {
         he_ctx_destroy(ctx);
         return HE_ENOMEM;
     }
-    *ctx->sh->dev_err = 0;
+    *ctx->sh->gave_up = 0;
     bool ok = cuda_ok(cudaMalloc(&ctx->d_mc, sizeof(ModConst) * LK)) && cuda_ok(cudaMalloc(&ctx->d_tw, tw.size() * 8)) &&
               cuda_ok(cudaMalloc(&ctx->d_fft, fft.size() * 4)) && cuda_ok(cudaMalloc(&ctx->d_sk, (size_t)LK * N * 8)) &&
               cuda_ok(cudaMalloc(&ctx->d_sk_mont, (size_t)LK * N * 8));
@@ -505,6 +505,8 @@ int he_ctx_fork(he_ctx *parent, void *stream, he_ctx **out) {
     for (int f = 0; f < HE_NTT_FORMS; ++f) ctx->ntt_form_ms[f] = parent->ntt_form_ms[f];
     ctx->d_bconv_a = parent->d_bconv_a;
     ctx->d_tc = parent->d_tc;
+    ctx->wait_limit = parent->wait_limit;
+    ctx->gave_up_seen = *static_cast<volatile unsigned int *>(ctx->sh->gave_up);
     ctx->bconv_a_off = parent->bconv_a_off;
     // the parent's pending work (keys, tables) must be complete before the fork's stream uses it
     if (cudaStreamSynchronize(parent->stream) != cudaSuccess) {
@@ -518,7 +520,15 @@ int he_ctx_fork(he_ctx *parent, void *stream, he_ctx **out) {
 int he_synchronize(he_ctx *ctx) {
     if (!ctx) return HE_EINVAL;
     const int rc = he_check(cudaStreamSynchronize(ctx->stream));
-    return rc == HE_OK && *ctx->sh->dev_err ? HE_ETIMEOUT : rc;
+    if (rc != HE_OK || !wait_gave_up(ctx)) return rc;
+    ctx->gave_up_seen = *static_cast<volatile unsigned int *>(ctx->sh->gave_up);
+    return HE_ETIMEOUT;
+}
+
+int he_set_wait_limit(he_ctx *ctx, int64_t polls) {
+    if (!ctx || polls < 0 || polls > HE_WAIT_LIMIT) return HE_EINVAL;
+    ctx->wait_limit = (unsigned int)polls;
+    return HE_OK;
 }
 
 int he_launch_count(const he_ctx *ctx, int64_t *count) {
@@ -651,6 +661,7 @@ int he_encrypt_dnonce(he_ctx *ctx, const he_pt *pt, const uint64_t *nonce_dev, h
 int he_decrypt(he_ctx *ctx, const he_ct *ct, double *slots_out) {
     if (!ctx || !ct || !ct->data || !slots_out) return HE_EINVAL;
     if (ct->level < 0 || ct->level >= ctx->L) return HE_ELEVEL;
+    if (wait_gave_up(ctx)) return HE_ETIMEOUT;
     if (launch_decrypt_slots(ctx, ct, slots_out)) return last_launch();
     double *coef = reinterpret_cast<double *>(ctx_scratch(ctx, ctx->n));
     if (!coef) return HE_ENOMEM;
@@ -1516,6 +1527,7 @@ int he_matmult_decrypt(he_ctx *ctx, const he_plan *plan, const he_ct *cts, int n
         if (cts[r].level < 0 || cts[r].level >= ctx->L) return HE_ELEVEL;
         if (cts[r].scale != cts[0].scale) return HE_ESCALE;
     }
+    if (wait_gave_up(ctx)) return HE_ETIMEOUT;
     if (launch_decrypt_ras(ctx, *plan, cts, n_ct, mask, y_out)) return last_launch();
     const size_t N = ctx->n;
     uint64_t *s = ctx_scratch(ctx, (size_t)n_ct * N + (size_t)n_ct * (N / 2));

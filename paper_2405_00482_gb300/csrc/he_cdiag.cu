@@ -329,11 +329,11 @@ int he_cdiag_matmult(he_ctx *ctx, const he_cdmat *W, const he_ct *cts, int n_ct,
     const int64_t K = W->K, N = ctx->n;
     for (int64_t k = 0; k < K; ++k)
         if (!outs[k].data) return HE_EINVAL;
+    if (W->tc.wt && wait_gave_up(ctx)) return HE_ETIMEOUT;
     const size_t w_pre = (size_t)K * 2 * nl * N, w_last = (size_t)K * 2 * N;
     uint64_t *pre = ctx_scratch(ctx, w_pre + w_last + (W->tc.wt ? cdiag_tc_words(ctx, n_ct, level) : 0));
     if (!pre) return HE_ENOMEM;
     uint64_t *last = pre + w_pre;
-    if (*ctx->sh->dev_err) return HE_ETIMEOUT;
     if (W->tc.wt) cdiag_tc_mac(ctx, &W->tc, cts, n_ct, level, K, pre, last + w_last);
     CtTable tab;
     for (int i = 0; i < n_ct; ++i) tab.p[i] = cts[i].data;
@@ -442,6 +442,7 @@ int he_cdiag_transpose(he_ctx *ctx, const he_ct *cts, int64_t m, int64_t n, he_c
 
 int he_cdiag_decode(he_ctx *ctx, int64_t m, int64_t n, int64_t K, const double *slots, double *Z) {
     if (!ctx || !slots || !Z || !pow2(m) || !pow2(n) || K < 1) return HE_EINVAL;
+    if (wait_gave_up(ctx)) return HE_ETIMEOUT;
     ctx->launches++;
     launch_k(cdiag_decode_kernel, blocks_for(m * K), 256, 0, ctx->stream, slots, m, n, K, ctx->n / 2, Z);
     return cudaGetLastError() == cudaSuccess ? HE_OK : HE_ECUDA;

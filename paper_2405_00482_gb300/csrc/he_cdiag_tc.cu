@@ -59,7 +59,6 @@ constexpr int TC_TR_WORDS = 32 * 17;        // a fold warp's transposition: 32 c
 constexpr int TC_SMEM = TC_STAGES * TC_STAGE_BYTES + TC_FOLD_WARPS * TC_TR_WORDS * 8 + 8 * (2 * TC_STAGES + 2 * TC_SLOTS) + 16;
 constexpr int TC_TMEM_COLS = TC_SLOTS * TC_ROWS;
 constexpr int TC_RES_THREADS = 512;         // residues kernel: thread (row, octet of a chunk)
-constexpr unsigned TC_WAIT_LIMIT = 1u << 21;  // polls of a barrier (each suspended for a while by the hardware) before giving up
 
 // per limb: the moduli count and the reconstruction constants
 struct TcLimb {
@@ -94,9 +93,10 @@ __constant__ TcTables c_tc = tc_tables();
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint32_t bar, int count) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory"); }
-// waits for the phase's completion, at most TC_WAIT_LIMIT polls; once a wait gave up (ok false) none waits
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, int parity, bool ok) {
-    for (unsigned n = 0; ok && n < TC_WAIT_LIMIT; ++n) {
+// waits for the phase's completion, at most `limit` polls (each suspended for a while by the hardware);
+// once a wait gave up (ok false) none waits
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, int parity, bool ok, unsigned limit) {
+    for (unsigned n = 0; ok && n < limit; ++n) {
         uint32_t done;
         asm volatile(
             "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
@@ -194,6 +194,7 @@ struct TcGeom {
     int32_t cnt, i0, nl, K, logn, lg_n, accumulate;
     int32_t first, tiles;          // this slice's tiles, numbered over (limb, row tile)
     int32_t chunks;                // 64-wide chunks of the longest window
+    uint32_t wait_limit;           // of the product kernel's waits (mbar_wait)
     int64_t tile_bytes;            // operand blocks of a tile: [modulus][chunk][64 rows x 128 bytes]
 };
 
@@ -285,7 +286,7 @@ __device__ __forceinline__ bool tc_fold(const TcGeom &g, const TcTile &t, int kb
     bool ok = true;
     for (int m = 0; m < lb.n_mod && ok; ++m, ++slot_it) {
         const uint32_t slot = slot_it % TC_SLOTS;
-        ok = mbar_wait(acc_full + 8 * slot, (int)((slot_it / TC_SLOTS) & 1), ok);
+        ok = mbar_wait(acc_full + 8 * slot, (int)((slot_it / TC_SLOTS) & 1), ok, g.wait_limit);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         float v[16];
         tmem_ld16(v, tmem + slot * TC_ROWS + (uint32_t)part * 16 + lanes);
@@ -343,7 +344,7 @@ __device__ __forceinline__ bool tc_fold(const TcGeom &g, const TcTile &t, int kb
 // orbit and nearly the same window), so the weights' blocks that each copies for itself come from L2.
 __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __grid_constant__ TcGeom g, const __grid_constant__ CdiagTc tc,
                                                                      const TcLimb *__restrict__ limbs, const unsigned char *__restrict__ X, uint64_t *pre,
-                                                                     const ModConst *__restrict__ mc, unsigned int *err) {
+                                                                     const ModConst *__restrict__ mc, unsigned int *gave_up) {
     HE_GRID_LAUNCH();
     extern __shared__ __align__(1024) unsigned char smem_tc[];  // the swizzle repeats every 1024 bytes
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem_tc + TC_STAGES * TC_STAGE_BYTES) + TC_FOLD_WARPS * TC_TR_WORDS;
@@ -387,7 +388,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
                 for (int m = 0; m < n_mod && ok; ++m)
                     for (int c = t.step0 / 4; c * 4 < t.step1 && ok; ++c, ++it) {
                         const uint32_t st = it % TC_STAGES;
-                        if (it >= TC_STAGES) ok = mbar_wait(empty + 8 * st, (int)((it / TC_STAGES - 1) & 1), ok);
+                        if (it >= TC_STAGES) ok = mbar_wait(empty + 8 * st, (int)((it / TC_STAGES - 1) & 1), ok, g.wait_limit);
                         if (!ok) break;
                         const uint32_t bar = full + 8 * st, A = full_stage + st * TC_STAGE_BYTES;
                         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(TC_STAGE_BYTES) : "memory");
@@ -403,7 +404,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
             // no copy may land after this CTA: where a wait gave up, here or in the other warps, nobody else
             // waits for the last ones (otherwise they are long complete)
             for (uint32_t i = it < TC_STAGES ? 0 : it - TC_STAGES; i < it; ++i)
-                if (!mbar_wait(full + 8 * (i % TC_STAGES), (int)((i / TC_STAGES) & 1), true)) ok = false;
+                if (!mbar_wait(full + 8 * (i % TC_STAGES), (int)((i / TC_STAGES) & 1), true, HE_WAIT_LIMIT)) ok = false;
         }
     } else if (warp == 1) {
         // products: the whole warp walks the rings, one elected lane issues, so that descriptors and
@@ -414,10 +415,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
             const int n_mod = limbs[t.u].n_mod;
             for (int m = 0; m < n_mod && ok; ++m, ++slot_it) {
                 const uint32_t slot = slot_it % TC_SLOTS, d = tmem + slot * TC_ROWS;
-                if (slot_it >= TC_SLOTS) ok = mbar_wait(acc_empty + 8 * slot, (int)((slot_it / TC_SLOTS - 1) & 1), ok);
+                if (slot_it >= TC_SLOTS) ok = mbar_wait(acc_empty + 8 * slot, (int)((slot_it / TC_SLOTS - 1) & 1), ok, g.wait_limit);
                 for (int c = t.step0 / 4; c * 4 < t.step1 && ok; ++c, ++it) {
                     const uint32_t st = it % TC_STAGES;
-                    ok = mbar_wait(full + 8 * st, (int)((it / TC_STAGES) & 1), ok);
+                    ok = mbar_wait(full + 8 * st, (int)((it / TC_STAGES) & 1), ok, g.wait_limit);
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t A = full_stage + st * TC_STAGE_BYTES;
@@ -436,7 +437,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
         // likewise the products: none may write tensor memory that has been given back
         if (elect_one()) umma_commit(drained);
         __syncwarp();
-        if (!mbar_wait(drained, 0, true)) ok = false;
+        if (!mbar_wait(drained, 0, true, HE_WAIT_LIMIT)) ok = false;
     } else {
         uint32_t slot_it = 0;
         uint64_t *tr = bars - (TC_FOLD_WARPS - (warp - 2)) * TC_TR_WORDS;
@@ -447,11 +448,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
             else ok = tc_fold<3>(g, t, unit / g.tiles, lb, mc[t.u], pre, tmem, acc_full, acc_empty, tr, slot_it);
         }
     }
-    if (!ok) atomicExch(err, 1u);
     // every copy and product is complete: the tensor memory is free
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncwarp();
-    __syncthreads();
+    if (__syncthreads_or(!ok) && threadIdx.x == 0) atomicAdd_system(gave_up, 1u);
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(TC_TMEM_COLS) : "memory");
 }
 
@@ -592,6 +592,7 @@ void cdiag_tc_mac(he_ctx *ctx, const CdiagTc *tc, const he_ct *cts, int n_ct, in
         g.logn = ctx->log_n;
         g.lg_n = tc->lg_n;
         g.accumulate = i0 > 0;
+        g.wait_limit = ctx->wait_limit;
         g.chunks = pass.chunks;
         g.tile_bytes = pass.tile_bytes;
         for (int i = 0; i < g.cnt; ++i) g.ct[i] = cts[i0 + i].data;
@@ -600,7 +601,7 @@ void cdiag_tc_mac(he_ctx *ctx, const CdiagTc *tc, const he_ct *cts, int n_ct, in
             ctx->launches += 2;
             launch_k(cdiag_tc_residues_kernel, dim3((unsigned)g.tiles, (unsigned)g.chunks), TC_RES_THREADS, 0, ctx->stream, g, limbs, X);
             launch_k(cdiag_tc_mma_kernel, std::min(ctx->sms, g.tiles * col_blocks), TC_THREADS, TC_SMEM, ctx->stream, g, *tc, limbs,
-                     (const unsigned char *)X, pre, (const ModConst *)ctx->d_mc, ctx->sh->dev_err);
+                     (const unsigned char *)X, pre, (const ModConst *)ctx->d_mc, ctx->sh->gave_up);
         }
     }
 }

@@ -74,7 +74,7 @@ int h2d(he_ctx *ctx, void *dst, const void *src, size_t bytes) {
 
 // device -> host on the context's stream.  Page-locked destination: one asynchronous copy, the
 // values valid once the stream reaches it.  Pageable: the call waits and the values are valid on
-// return.
+// return (HE_ETIMEOUT if a kernel's bounded wait had given up by then).
 int d2h(he_ctx *ctx, void *dst, const void *src, size_t bytes) {
     if (bytes == 0) return HE_OK;
     if (page_locked(dst)) return he_check(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, ctx->stream));
@@ -84,7 +84,7 @@ int d2h(he_ctx *ctx, void *dst, const void *src, size_t bytes) {
     if (cudaMemcpyAsync(h, src, bytes, cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess) return HE_ECUDA;
     if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return HE_ECUDA;
     memcpy(dst, h, bytes);
-    return HE_OK;
+    return wait_gave_up(ctx) ? HE_ETIMEOUT : HE_OK;
 }
 
 // serialized ciphertext: header, the primes of its level, then [2][level+1][N] canonical
@@ -189,7 +189,7 @@ int he_ct_export_host(he_ctx *ctx, const he_ct *ct, void *buf, size_t *len) {
     // the bytes are complete on return, whatever memory they are in
     if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return HE_ECUDA;
     *len = need;
-    return HE_OK;
+    return wait_gave_up(ctx) ? HE_ETIMEOUT : HE_OK;
 }
 
 int he_ct_host_level(const void *buf, size_t len, int32_t *level) {

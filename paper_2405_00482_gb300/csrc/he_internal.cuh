@@ -171,11 +171,11 @@ struct he_shared {
     int key_fusion = 1;                       // fused key tables of encoded matrices: 0 never, 1 on reuse, 2 always
     size_t fuse_max = (size_t)8 << 30;        // largest fused table built (bytes)
     void *owned[7] = {};                      // device tables: d_mc, d_tw, d_fft, d_sk, d_sk_mont, d_bconv_a, d_tc
-    unsigned int *dev_err = nullptr;          // page-locked: set by a kernel whose bounded wait gave up
+    unsigned int *gave_up = nullptr;          // page-locked: CTAs whose bounded wait gave up, counted by the kernels
     ~he_shared() {
         for (auto &kv : keys) cudaFree(kv.second);
         for (void *p : owned) cudaFree(p);
-        cudaFreeHost(dev_err);
+        cudaFreeHost(gave_up);
     }
     uint64_t *key(uint32_t g) {
         std::lock_guard<std::mutex> lock(mu);
@@ -184,6 +184,7 @@ struct he_shared {
     }
 };
 
+#define HE_WAIT_LIMIT (1u << 21)
 struct he_ctx {
     int log_n, n, L, K, dnum, alpha;
     int device;                       // CUDA device the context was created on (current at he_ctx_create)
@@ -223,6 +224,8 @@ struct he_ctx {
     void *stage_host = nullptr;
     size_t stage_host_bytes = 0;
     cudaEvent_t stage_ev = nullptr;
+    unsigned int gave_up_seen = 0;           // the family's count of waits given up when he_synchronize last returned
+    unsigned int wait_limit = HE_WAIT_LIMIT;  // polls of a barrier before a kernel's wait gives up (he_set_wait_limit)
     // kernels launched so far, and CUDA-event timing of the MatMult loop kernel when enabled
     int64_t launches;
     bool prof_on;
@@ -253,6 +256,10 @@ inline void each_logn(F f) {
 // contexts of one family (a context and its forks) share tables and keys, so plaintext
 // matrices made on one serve all
 inline bool same_family(const he_ctx *a, const he_ctx *b) { return a == b || (a && b && a->sh && a->sh == b->sh); }
+
+// a bounded wait of some kernel of the family gave up since this context last reported it
+// (he_synchronize): the calls that hand out or consume such results return HE_ETIMEOUT
+inline bool wait_gave_up(const he_ctx *ctx) { return *static_cast<const volatile unsigned int *>(ctx->sh->gave_up) != ctx->gave_up_seen; }
 
 // one MatMult of a batch (device table entry)
 struct MMJob {

@@ -49,6 +49,7 @@ _SIGS = {
     "he_ctx_destroy": (None, [_vp]),
     "he_ctx_fork": (ctypes.c_int, [_vp, _vp, ctypes.POINTER(_vp)]),
     "he_synchronize": (ctypes.c_int, [_vp]),
+    "he_set_wait_limit": (ctypes.c_int, [_vp, _i64]),
     "he_ctx_info": (ctypes.c_int, [_vp, ctypes.POINTER(_i64), ctypes.POINTER(_i32), ctypes.POINTER(_i32)]),
     "he_keygen": (ctypes.c_int, [_vp, ctypes.POINTER(_i32), ctypes.c_int]),
     "he_launch_count": (ctypes.c_int, [_vp, ctypes.POINTER(_i64)]),
@@ -513,6 +514,10 @@ class Context:
 
     def synchronize(self):
         _check(_lib().he_synchronize(self.handle), "he_synchronize")
+
+    def set_wait_limit(self, polls: int = 1 << 21):
+        """Polls after which a kernel's bounded wait gives up (he_set_wait_limit)."""
+        _check(_lib().he_set_wait_limit(self.handle, polls), "he_set_wait_limit")
 
     def launch_count(self) -> int:
         v = _i64()
