@@ -743,14 +743,15 @@ int he_rotate_hoisted(he_ctx *ctx, const he_ct *in, const int32_t *steps, int k,
             return HE_ECUDA;
     const int n_jobs = (int)jobs.size();
     if (n_jobs > 0) {
-        // one ModUp of c1 (O4), then the key switch of every rotation, two launches per 128
+        // one ModUp of c1 (O4), then the key switch of every rotation, two or four launches per chunk
         const ModUpConst &mu = ctx->modup[level];
-        const size_t wD = (size_t)mu.ndig * mu.ext * N, wc = nl * N, wp = keyswitch_many_pc_words(ctx, n_jobs);
-        uint64_t *s = ctx_scratch(ctx, wD + wc + wp);
+        const size_t wD = (size_t)mu.ndig * mu.ext * N, wc = nl * N, wp = keyswitch_pc_words(ctx);
+        int chunk;
+        uint64_t *s = chunk_scratch(ctx, n_jobs, [&](int c) { return wD + wc + c * wp; }, &chunk);
         if (!s) return HE_ENOMEM;
         uint64_t *D = s, *coef = D + wD, *pc = coef + wc;
         launch_modup(ctx, in->data + nl * N, level, D, coef);
-        launch_keyswitch_many(ctx, jobs.data(), n_jobs, level, D, 0, pc);
+        launch_keyswitch_many(ctx, jobs.data(), n_jobs, level, D, 0, pc, chunk);
     }
     for (int i = 0; i < k; ++i) {
         outs[i].level = level;
@@ -789,10 +790,10 @@ int he_rotate_many(he_ctx *ctx, const he_ct *ins, const int32_t *steps, int coun
     }
     const int n_jobs = (int)jobs.size();
     if (n_jobs > 0) {
-        // chunks of HE_ROT_CHUNK rotations, their job tables passed as kernel parameters; the
+        // chunks of up to HE_ROT_CHUNK rotations, their job tables passed as kernel parameters; the
         // chunks reuse one scratch region in stream order
-        const int chunk = n_jobs < HE_ROT_CHUNK ? n_jobs : HE_ROT_CHUNK;
-        uint64_t *s = ctx_scratch(ctx, (size_t)chunk * rotate_many_words(ctx, level));
+        int chunk;
+        uint64_t *s = chunk_scratch(ctx, n_jobs, [&](int c) { return c * rotate_many_words(ctx, level); }, &chunk);
         if (!s) return HE_ENOMEM;
         for (int c0 = 0; c0 < n_jobs; c0 += chunk) launch_rotate_many(ctx, jobs.data() + c0, std::min(chunk, n_jobs - c0), level, s);
     }

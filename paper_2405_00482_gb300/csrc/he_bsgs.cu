@@ -12,6 +12,7 @@
 // over g is rescaled once.  Galois keys: B - 1 + G - 1 instead of m' - 1.  Every step is the
 // exact modular arithmetic of the corresponding O1-O4, so the output is bit-identical to their
 // composition in that order.
+#include <algorithm>
 #include <vector>
 
 #include "he_internal.cuh"
@@ -98,12 +99,14 @@ int matmult_bsgs(he_ctx *ctx, he_ptmat *pm, const he_ct *ins, he_ct *outs) {
     }
     // scratch: baby rotations, ModUp digits and c1 coefficients of one input, the key switch's
     // tables, partial sums, giant rotations and their batch scratch, rescale temporaries
-    const int gchunk = G - 1 < HE_ROT_CHUNK ? G - 1 : HE_ROT_CHUNK;
-    const size_t wX = (size_t)C * B * ct_w, wD = (size_t)mu.ndig * mu.ext * N + nl * N, wpc = B > 1 ? keyswitch_many_pc_words(ctx, B - 1) : 0,
-                 wI = (size_t)G * ct_w, wRot = (size_t)(G - 1) * ct_w, wRm = gchunk > 0 ? (size_t)gchunk * rotate_many_words(ctx, level) : 0,
+    const size_t wX = (size_t)C * B * ct_w, wD = (size_t)mu.ndig * mu.ext * N + nl * N, wI = (size_t)G * ct_w, wRot = (size_t)(G - 1) * ct_w,
                  wT = 2 * (size_t)(ctx->K > 1 ? ctx->K : 1) * N + 2 * N;
-    uint64_t *s = ctx_scratch(ctx, wX + wD + wpc + wI + wRot + wRm + wT);
+    auto w_pc = [&](int c) { return (size_t)std::min(B - 1, c) * keyswitch_pc_words(ctx); };
+    auto w_rm = [&](int c) { return (size_t)std::min(G - 1, c) * rotate_many_words(ctx, level); };
+    int chunk;
+    uint64_t *s = chunk_scratch(ctx, std::max(B, G) - 1, [&](int c) { return wX + wD + w_pc(c) + wI + wRot + w_rm(c) + wT; }, &chunk);
     if (!s) return HE_ENOMEM;
+    const size_t wpc = w_pc(chunk), wRm = w_rm(chunk);
     uint64_t *X = s, *D = X + wX, *coef = D + (size_t)mu.ndig * mu.ext * N, *pc = D + wD, *inner = pc + wpc, *rot = inner + wI, *rm = rot + wRot,
              *tmp = rm + wRm;
     // baby steps: x_{c,0} = ct_c, x_{c,b} = RotL(ct_c, b) with one decomposition per input
@@ -114,7 +117,7 @@ int matmult_bsgs(he_ctx *ctx, he_ptmat *pm, const he_ct *ins, he_ct *outs) {
         std::vector<RotJob> jobs(B - 1);
         for (int b = 1; b < B; ++b) jobs[b - 1] = RotJob{ins[c].data, Xc + (size_t)b * ct_w, kb[b], gb[b], 0};
         launch_modup(ctx, ins[c].data + nl * N, level, D, coef);
-        launch_keyswitch_many(ctx, jobs.data(), B - 1, level, D, 0, pc);
+        launch_keyswitch_many(ctx, jobs.data(), B - 1, level, D, 0, pc, chunk);
     }
     const unsigned eb = (unsigned)((N + 255) / 256);
     for (int r = 0; r < R; ++r) {
@@ -129,8 +132,8 @@ int matmult_bsgs(he_ctx *ctx, he_ptmat *pm, const he_ct *ins, he_ct *outs) {
         ctx->launches++;
         launch_k(bsgs_mac_kernel, dim3(eb, (unsigned)nl, (unsigned)G), 256, 0, ctx->stream, bg, (const ModConst *)ctx->d_mc, ctx->log_n);
         // giant steps RotL(s_g, g B), g >= 1, as batches of O3 on different ciphertexts
-        for (int g0 = 1; g0 < G; g0 += HE_ROT_CHUNK) {
-            const int n = G - g0 < HE_ROT_CHUNK ? G - g0 : HE_ROT_CHUNK;
+        for (int g0 = 1; g0 < G; g0 += chunk) {
+            const int n = G - g0 < chunk ? G - g0 : chunk;
             std::vector<RotJob> jobs(n);
             for (int t = 0; t < n; ++t) {
                 const int g = g0 + t;

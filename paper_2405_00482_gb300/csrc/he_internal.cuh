@@ -350,7 +350,7 @@ struct he_batch {
 int launch_matmult_batch(he_ctx *ctx, he_batch *b, cudaStream_t stream);
 // words of scratch per rotation job at `level`, and the launches of `count` jobs (device table)
 size_t rotate_many_words(const he_ctx *ctx, int level);
-// count <= HE_ROT_CHUNK jobs (host table), scratch of count rotate_many_words
+// count <= HE_ROT_CHUNK jobs (host table), scratch of count * rotate_many_words
 void launch_rotate_many(he_ctx *ctx, const RotJob *jobs, int count, int level, uint64_t *scratch);
 // ModUp with the INT8 tensor-core basis extension (he_bconv.cu): for jobs j < count, c1 of job j
 // in NTT form (jobs[j].ct + (level+1) N when jobs is given, else c1_ntt) and in coefficient form
@@ -361,10 +361,10 @@ void launch_modup_i8(he_ctx *ctx, const RotTable *jobs, int count, int level, co
 int bconv_i8_tables(he_ctx *ctx);
 // key switch (inner product, ModDown, automorphism of c0) of `count` rotations (host table) whose
 // ModUp digits are at D + j d_stride (d_stride 0: one shared decomposition), two (few rotations)
-// or four launches per HE_ROT_CHUNK rotations; pc: scratch of keyswitch_many_pc_words(ctx, count)
-// words, laid out [min(count, HE_ROT_CHUNK)][2][K][N] then [..][2][level+1][N]
-size_t keyswitch_many_pc_words(const he_ctx *ctx, int count);
-void launch_keyswitch_many(he_ctx *ctx, const RotJob *jobs, int count, int level, const uint64_t *D, int64_t d_stride, uint64_t *pc);
+// or four launches per `chunk` (<= HE_ROT_CHUNK) rotations; pc: scratch of chunk * keyswitch_pc_words(ctx)
+// words, laid out [chunk][2][K][N] then [chunk][2][level+1][N]
+size_t keyswitch_pc_words(const he_ctx *ctx);
+void launch_keyswitch_many(he_ctx *ctx, const RotJob *jobs, int count, int level, const uint64_t *D, int64_t d_stride, uint64_t *pc, int chunk);
 int mm_variant_count();
 int mm_variant_tile(int v);  // coefficients per tile of loop-kernel variant v
 void mm_variant_shape(int v, int *vec, int *grp, int *stages, int *ga);
@@ -372,6 +372,20 @@ int mm_batch_ctas_per_sm(int v, int ndig);
 int tune_matmult_loop(he_ctx *ctx, he_ptmat *pm, const uint64_t *ct, const uint64_t *D, uint64_t *acc, uint64_t *cacc, bool rows);
 int tune_matmult_fused(he_ctx *ctx, he_ptmat *pm, const uint64_t *ct, const uint64_t *D, uint64_t *acc, uint64_t *cacc);
 bool capturing(cudaStream_t st);           // st is being captured into a graph
+uint64_t *ctx_scratch(he_ctx *ctx, size_t words);  // nullptr on allocation failure
+// Scratch of a call that takes `count` rotations in chunks, words(c) for chunks of c; the chunk goes to
+// *chunk.  HE_ROT_CHUNK at a time, or 64 or 32 where that much scratch cannot be had: no memory (a chunk
+// of 128 on the widest ring at N = 2^14 takes 4.3 GB), or a stream under capture, where it cannot grow.
+template <class W>
+inline uint64_t *chunk_scratch(he_ctx *ctx, int count, W words, int *chunk) {
+    for (int c = count < HE_ROT_CHUNK ? count : HE_ROT_CHUNK;; c = c > 64 ? 64 : 32) {
+        *chunk = c;
+        if (c > 32 && words(c) > ctx->scratch_words && capturing(ctx->stream)) continue;
+        uint64_t *s = ctx_scratch(ctx, words(c));
+        if (s || c <= 32) return s;
+        cudaGetLastError();
+    }
+}
 bool mm_variant_fusable(int v, int ndig);  // variant v has a fused-key form for ndig digits
 void launch_fuse_keys(he_ctx *ctx, he_ptmat *pm);  // pm->fused from pm->data and the bound Galois keys
 // defined in he_api.cu (inside its extern "C" block)
@@ -445,7 +459,6 @@ inline cudaError_t launch_cluster(void (*kernel)(KArgs...), int grid, int block,
 int he_check(cudaError_t e);
 // Galois element 5^r mod 2N of a left rotation by `step` slots, r = step mod N/2 in [0, N/2)
 uint32_t galois_of(const he_ctx *ctx, int64_t step);
-uint64_t *ctx_scratch(he_ctx *ctx, size_t words);  // nullptr on allocation failure
 
 // NTT of `groups` x map.n limb-polys; in and out may alias.
 void launch_from_mont(he_ctx *ctx, const uint64_t *data, uint64_t *out, int groups, const LimbMap &map);

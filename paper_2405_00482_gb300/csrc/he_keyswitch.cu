@@ -15,6 +15,8 @@
 // small) and stream the keys from HBM.  Each thread forms KS_U coefficients at once with every
 // load of those coefficients (all digits when their count is known at compile time) issued
 // before the first product, so a thread's loads overlap instead of queueing one after another.
+#include <algorithm>
+
 #include "he_internal.cuh"
 #include "he_ntt.cuh"
 
@@ -393,23 +395,22 @@ auto ks_pick(int logn, int ndig, F f) {
 
 }  // namespace
 
-size_t keyswitch_many_pc_words(const he_ctx *ctx, int count) {
-    const int c = count < HE_ROT_CHUNK ? count : HE_ROT_CHUNK;
-    return (size_t)c * 2 * (ctx->K + ctx->L) * ctx->n;  // pc [c][2][K][N], then cv [c][2][nl][N] (nl <= L)
+size_t keyswitch_pc_words(const he_ctx *ctx) {
+    return 2 * (size_t)(ctx->K + ctx->L) * ctx->n;  // pc [2][K][N] and cv [2][nl][N] (nl <= L)
 }
 
-void launch_keyswitch_many(he_ctx *ctx, const RotJob *jobs, int count, int level, const uint64_t *D, int64_t d_stride, uint64_t *pc) {
+void launch_keyswitch_many(he_ctx *ctx, const RotJob *jobs, int count, int level, const uint64_t *D, int64_t d_stride, uint64_t *pc, int chunk) {
     const ModUpConst &mu = ctx->modup[level];
     const ModDownConst &md = ctx->moddown[level];
     const int logn = ctx->log_n;
     cudaStream_t st = ctx->stream;
     const uint64_t *tw = ctx->d_tw;
     const ModConst *mc = ctx->d_mc;
-    const int cmax = count < HE_ROT_CHUNK ? count : HE_ROT_CHUNK;
+    const int cmax = count < chunk ? count : chunk;
     uint64_t *cv = pc + (size_t)cmax * 2 * ctx->K * ctx->n;  // [cmax][2][level+1][N] after pc [cmax][2][K][N]
     // one chunk's launches with transform variant v (0: ntt_threads per CTA, 1: 512 threads,
     // 2: two phases of small CTAs per transform), of at most nmax rotations
-    auto issue = [&](int c0, int v, int nmax = HE_ROT_CHUNK) {
+    auto issue = [&](int c0, int v, int nmax) {
         const int n = count - c0 < nmax ? count - c0 : nmax;
         RotTable tab{};
         for (int j = 0; j < n; ++j) tab.j[j] = jobs[c0 + j];
@@ -493,7 +494,7 @@ void launch_keyswitch_many(he_ctx *ctx, const RotJob *jobs, int count, int level
                 float ms = 1e30f;
                 for (int rep = 0; rep < 3; ++rep) {
                     cudaEventRecord(e0, st);
-                    issue(0, v, 64);
+                    issue(0, v, std::min(cmax, 64));
                     cudaEventRecord(e1, st);
                     if (cudaEventSynchronize(e1) != cudaSuccess) break;
                     float t = 0.0f;
@@ -508,7 +509,7 @@ void launch_keyswitch_many(he_ctx *ctx, const RotJob *jobs, int count, int level
         if (e0) cudaEventDestroy(e0);
         if (e1) cudaEventDestroy(e1);
     }
-    for (int c0 = 0; c0 < count; c0 += HE_ROT_CHUNK) issue(c0, ctx->ks_variant < 0 ? 0 : ctx->ks_variant);
+    for (int c0 = 0; c0 < count; c0 += cmax) issue(c0, ctx->ks_variant < 0 ? 0 : ctx->ks_variant, cmax);
 }
 
 void keyswitch_set_smem_limits(int max_bytes) {

@@ -2309,7 +2309,7 @@ void launch_rotate_many(he_ctx *ctx, const RotJob *jobs, int count, int level, u
         launch_cluster(by_logn(ctx->log_n, [](auto L) { return rot_modup_cl_kernel<L.value>; }), items * HE_NTT_CL_SIZE, cl_threads(ctx->log_n),
                        cl_fused_smem_bytes(ctx->log_n), st, tab, rg, mu, (const uint64_t *)ctx->d_tw, (const ModConst *)ctx->d_mc, ctx->log_n);
         ctx->launches++;
-        launch_keyswitch_many(ctx, jobs, count, level, rg.D, rg.d_w, rg.pcoef);
+        launch_keyswitch_many(ctx, jobs, count, level, rg.D, rg.d_w, rg.pcoef, count);
         return;
     }
     if (ctx->bconv != HE_BCONV_INT8_TC && use_two_phase(ctx, items)) {
@@ -2327,7 +2327,7 @@ void launch_rotate_many(he_ctx *ctx, const RotJob *jobs, int count, int level, u
         else if (ctx->log_n == 13) go(std::integral_constant<int, 13>{}, std::integral_constant<int, 4>{});
         else go(std::integral_constant<int, 14>{}, std::integral_constant<int, 4>{});
         ctx->launches += 4;
-        launch_keyswitch_many(ctx, jobs, count, level, rg.D, rg.d_w, rg.pcoef);
+        launch_keyswitch_many(ctx, jobs, count, level, rg.D, rg.d_w, rg.pcoef, count);
         return;
     }
     launch_k(rot_intt_c1_kernel, count * rg.nl, thr, smem, st, tab, rg, ctx->d_tw, ctx->d_mc, ctx->log_n);
@@ -2338,7 +2338,7 @@ void launch_rotate_many(he_ctx *ctx, const RotJob *jobs, int count, int level, u
         launch_k(rot_modup_kernel, count * mu.ndig * mu.ext, thr, smem, st, tab, rg, mu, ctx->d_tw, ctx->d_mc, ctx->log_n);
         ctx->launches++;
     }
-    launch_keyswitch_many(ctx, jobs, count, level, rg.D, rg.d_w, rg.pcoef);
+    launch_keyswitch_many(ctx, jobs, count, level, rg.D, rg.d_w, rg.pcoef, count);
 }
 
 void ops_set_smem_limits(int max_bytes) {
