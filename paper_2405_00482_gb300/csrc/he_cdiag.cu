@@ -21,19 +21,25 @@
 #define CD_WARPS 8     // warps per block (two coefficients each)
 #define CD_MAX_IN 1024 // ciphertexts per launch (kernel-parameter table)
 #define CD_MAX_OUT 512 // outputs per rescale launch
-// Weight columns from which he_cdiag_encode_weights lays the weights out for the tensor cores (rings
-// of 2^12 to 2^14, primes below 2^60, at least 8 weight rows: cdiag_tc_supported).  The integer form
-// takes the same time for 1 as for 128 columns; at 8 columns and 256 / 64 / 32 diagonals of N = 2^14
-// the whole call takes 1.16 / 0.65 / 0.65 ms on the tensor cores, 6.27 / 1.67 / 0.90 ms without.
+// The tensor cores (rings of 2^12 to 2^14, primes below 2^60: cdiag_tc_supported) take products of at
+// least 20 diagonals by at least 8 columns.  Their time hardly depends on the diagonals up to a window of
+// 64, that of the integer form is proportional to them and the same for 1 as for 128 columns.  The whole
+// call, tensor cores / integer form, in us for 2, 8, 16, 20, 24, 32 and 64 diagonals:
+//   N = 2^12,    8 columns, n =   64:    60/41   62/52   63/67   63/74   64/82   65/97   68/154
+//   N = 2^13,   16 columns, n =  256:   152/63  157/94 157/135 161/154 162/175 164/217  178/394
+//   N = 2^13,    8 columns, n = 4096:  186/82 189/112 194/155 199/173 204/194 214/235  268/400
+//   N = 2^14,    8 columns, n =   64: 476/162 488/302 497/505 506/601 515/695 525/890 558/1660
+//   N = 2^14,  128 columns, n =  256: 844/587 863/748 877/970 881/1078 882/1186 891/1406 928/2279
 #define CD_TC_MIN_COLS 8
+#define CD_TC_MIN_DIAGS 20
 
 struct he_cdmat {
     he_ctx *ctx;
     int64_t n, K;  // rows of W (= columns of A), columns of W
     int level;
     double scale;
-    uint64_t *pt;  // [level+1][N][K], NTT + Montgomery form; null when tc holds the weights
-    CdiagTc tc;    // the tensor-core form (he_cdiag_tc.cu)
+    uint64_t *pt;  // [level+1][N][K], NTT + Montgomery form
+    CdiagTc tc;    // the tensor-core form besides (he_cdiag_tc.cu), where products may take it
 };
 
 namespace {
@@ -249,8 +255,7 @@ int he_cdiag_encode_weights(he_ctx *ctx, const double *W, int64_t n, int64_t K, 
     cm->K = K;
     cm->level = level;
     cm->scale = (double)ctx->primes[level];
-    const bool tc = K >= CD_TC_MIN_COLS && cdiag_tc_supported(ctx, level, n);
-    if (!tc && cudaMalloc(&cm->pt, (size_t)nl * N * K * 8) != cudaSuccess) {
+    if (cudaMalloc(&cm->pt, (size_t)nl * N * K * 8) != cudaSuccess) {
         delete cm;
         return HE_ENOMEM;
     }
@@ -268,16 +273,17 @@ int he_cdiag_encode_weights(he_ctx *ctx, const double *W, int64_t n, int64_t K, 
     ctx->launches += 3;
     launch_k(cdiag_weights_kernel, blocks_for(K * (N / 2)), 256, 0, ctx->stream, W, n, K, N / 2, slots);
     launch_encode(ctx, slots, N / 2, N / 2, (int)K, cm->scale, coef);
-    launch_ntt_from_int64(ctx, coef, cols, (int)K, m, tc ? 0 : 1);
-    int rc = HE_OK;
-    if (tc)
-        rc = cdiag_tc_prepare(ctx, &cm->tc, n, K, level, cols);
-    else
-        launch_k(transpose_cols_kernel, blocks_for(K * nl * N), 256, 0, ctx->stream, cols, cm->pt, (int)K, (int)nl, ctx->log_n);
-    if (cudaGetLastError() != cudaSuccess && rc == HE_OK) rc = HE_ECUDA;
-    if (rc != HE_OK) {
+    launch_ntt_from_int64(ctx, coef, cols, (int)K, m, 1);
+    launch_k(transpose_cols_kernel, blocks_for(K * nl * N), 256, 0, ctx->stream, cols, cm->pt, (int)K, (int)nl, ctx->log_n);
+    bool ok = cudaGetLastError() == cudaSuccess;
+    // the weights' residues pad the columns to 128: without memory for them the integer form serves
+    if (K >= CD_TC_MIN_COLS && n >= CD_TC_MIN_DIAGS && cdiag_tc_supported(ctx, level)) {
+        const bool prepared = cdiag_tc_prepare(ctx, &cm->tc, n, K, level, cols);
+        ok = ok && (cudaGetLastError() == cudaSuccess || !prepared);
+    }
+    if (!ok) {
         he_cdmat_free(cm);
-        return rc;
+        return HE_ECUDA;
     }
     *out = cm;
     return HE_OK;
@@ -329,16 +335,25 @@ int he_cdiag_matmult(he_ctx *ctx, const he_cdmat *W, const he_ct *cts, int n_ct,
     const int64_t K = W->K, N = ctx->n;
     for (int64_t k = 0; k < K; ++k)
         if (!outs[k].data) return HE_EINVAL;
-    if (W->tc.wt && wait_gave_up(ctx)) return HE_ETIMEOUT;
+    bool tc = W->tc.wt && n_ct >= CD_TC_MIN_DIAGS;
+    if (tc && wait_gave_up(ctx)) return HE_ETIMEOUT;
     const size_t w_pre = (size_t)K * 2 * nl * N, w_last = (size_t)K * 2 * N;
-    uint64_t *pre = ctx_scratch(ctx, w_pre + w_last + (W->tc.wt ? cdiag_tc_words(ctx, n_ct, level) : 0));
+    // the integer form where the operands' scratch cannot be had: no memory, or a stream under capture
+    const size_t w_tc = tc ? cdiag_tc_words(ctx, n_ct, level) : 0;
+    if (w_pre + w_last + w_tc > ctx->scratch_words && capturing(ctx->stream)) tc = false;
+    uint64_t *pre = tc ? ctx_scratch(ctx, w_pre + w_last + w_tc) : nullptr;
+    if (!pre) {
+        cudaGetLastError();
+        tc = false;
+        pre = ctx_scratch(ctx, w_pre + w_last);
+    }
     if (!pre) return HE_ENOMEM;
     uint64_t *last = pre + w_pre;
-    if (W->tc.wt) cdiag_tc_mac(ctx, &W->tc, cts, n_ct, level, K, pre, last + w_last);
+    if (tc) cdiag_tc_mac(ctx, &W->tc, cts, n_ct, level, K, pre, last + w_last);
     CtTable tab;
     for (int i = 0; i < n_ct; ++i) tab.p[i] = cts[i].data;
     const int kmax = 16 * CD_COLS;  // columns per launch (16 lanes)
-    for (int64_t kb = 0; kb < K && !W->tc.wt; kb += kmax) {
+    for (int64_t kb = 0; kb < K && !tc; kb += kmax) {
         const dim3 grid((unsigned)(N / (2 * CD_WARPS)), (unsigned)nl);
         ctx->launches++;
         launch_k(cdiag_mac_kernel, grid, CD_WARPS * 32, 0, ctx->stream, tab, n_ct, nl, W->pt, (int)K, (int)kb, pre, ctx->d_mc, ctx->log_n);

@@ -458,20 +458,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
 // The weights' residues (W_k(block s) centred) (P/p_i)^-1 mod p_i, centred, as bfloat16, in blocks
 // [limb][modulus][orbit][128 columns][64 indices s] laid out as the tensor instruction reads them
 // (rows of 128 bytes, swizzled); s runs over a period n (at least 64: shorter periods repeat),
-// columns past K are zero.  cols: the encoded columns [K][nl][N], NTT form.
+// columns past K are zero.  cols: the encoded columns [K][nl][N], NTT and Montgomery form.
 __global__ void __launch_bounds__(256) cdiag_tc_weights_kernel(const uint64_t *__restrict__ cols, int K, int nl, int logn, const TcLimb *__restrict__ limbs,
                                                                const __grid_constant__ CdiagTc tc, const ModConst *__restrict__ mc) {
     HE_GRID_DEP();
     const int N = 1 << logn, n = 1 << tc.lg_n, lg_p = logn - 1 - tc.lg_n, wchunks = gridDim.x;
     const int orbit = blockIdx.y & 1, u = blockIdx.y >> 1, kb = blockIdx.z;
     const TcLimb &lb = limbs[u];
-    const uint64_t q = mc[u].q;
+    const uint64_t q = mc[u].q, qinv = mc[u].qinv;
     const int s = threadIdx.x & 63;
     const int at = block_first((blockIdx.x * TC_KC + s) & (n - 1), orbit, logn, lg_p);
     unsigned char *o = tc.wt + (tc.block[u] + ((int64_t)orbit * gridDim.z + kb) * wchunks + blockIdx.x) * TC_A_BYTES + 2 * (s & 7);
     for (int c = threadIdx.x >> 6; c < TC_COLS; c += 4) {
         const int k = kb * TC_COLS + c;
-        const uint64_t x = k < K ? cols[((int64_t)k * nl + u) * N + at] : 0;
+        const uint64_t x = k < K ? redc(0, cols[((int64_t)k * nl + u) * N + at], q, qinv) : 0;
         const bool neg = x > q / 2;
         float a[5];
         split14<5>(a, neg ? q - x : x);
@@ -506,8 +506,8 @@ void digits20(int32_t (&d)[3], uint64_t v, uint64_t q, int nd) {
 
 }  // namespace
 
-bool cdiag_tc_supported(const he_ctx *ctx, int level, int64_t n) {
-    if (ctx->log_n < 12 || ctx->log_n > 14 || n < 8) return false;
+bool cdiag_tc_supported(const he_ctx *ctx, int level) {
+    if (ctx->log_n < 12 || ctx->log_n > 14) return false;
     for (int u = 0; u <= level; ++u)
         if (!tc_moduli(ctx->primes[u])) return false;
     return true;
@@ -547,7 +547,7 @@ int cdiag_tc_tables(he_ctx *ctx) {
     return he_check(cudaMemcpy(d, limbs.data(), sizeof(TcLimb) * ctx->L, cudaMemcpyHostToDevice));
 }
 
-int cdiag_tc_prepare(he_ctx *ctx, CdiagTc *tc, int64_t n, int64_t K, int level, const uint64_t *cols) {
+bool cdiag_tc_prepare(he_ctx *ctx, CdiagTc *tc, int64_t n, int64_t K, int level, const uint64_t *cols) {
     const int nl = level + 1;
     tc->lg_n = 0;
     while (((int64_t)1 << tc->lg_n) < n) ++tc->lg_n;
@@ -557,11 +557,14 @@ int cdiag_tc_prepare(he_ctx *ctx, CdiagTc *tc, int64_t n, int64_t K, int level, 
         tc->block[u] = blocks;
         blocks += (int64_t)tc_moduli(ctx->primes[u]) * 2 * col_blocks * wchunks;
     }
-    if (cudaMalloc(&tc->wt, (size_t)blocks * TC_A_BYTES) != cudaSuccess) return HE_ENOMEM;
+    if (cudaMalloc(&tc->wt, (size_t)blocks * TC_A_BYTES) != cudaSuccess) {
+        tc->wt = nullptr;
+        return false;
+    }
     ctx->launches++;
     launch_k(cdiag_tc_weights_kernel, dim3((unsigned)wchunks, (unsigned)(2 * nl), (unsigned)col_blocks), 256, 0, ctx->stream, cols, (int)K, nl, ctx->log_n,
              (const TcLimb *)ctx->d_tc, *tc, (const ModConst *)ctx->d_mc);
-    return HE_OK;
+    return true;
 }
 
 void cdiag_tc_free(CdiagTc *tc) {

@@ -13,9 +13,10 @@ struct CdiagTc {
 };
 
 int cdiag_tc_tables(he_ctx *ctx);  // at context creation
-bool cdiag_tc_supported(const he_ctx *ctx, int level, int64_t n);
-// tc from the encoded columns (device, [K][level+1][N], NTT form, canonical)
-int cdiag_tc_prepare(he_ctx *ctx, CdiagTc *tc, int64_t n, int64_t K, int level, const uint64_t *cols);
+bool cdiag_tc_supported(const he_ctx *ctx, int level);
+// tc, for weights of n >= 8 rows, from the encoded columns (device, [K][level+1][N], NTT and Montgomery
+// form); false without memory for it
+bool cdiag_tc_prepare(he_ctx *ctx, CdiagTc *tc, int64_t n, int64_t K, int level, const uint64_t *cols);
 void cdiag_tc_free(CdiagTc *tc);
 // pre [K][2][level+1][N] = the products' sums over the n_ct ciphertexts; scratch: cdiag_tc_words
 void cdiag_tc_mac(he_ctx *ctx, const CdiagTc *tc, const he_ct *cts, int n_ct, int level, int64_t K, uint64_t *pre, uint64_t *scratch);
