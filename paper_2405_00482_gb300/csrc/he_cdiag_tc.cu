@@ -269,10 +269,18 @@ __global__ void __launch_bounds__(TC_RES_THREADS, 2) cdiag_tc_residues_kernel(co
     else tc_residues<5>(g, t, lb.n_mod, ct, out);
 }
 
+// the limit of the product kernel's waits: a constant unless he_set_wait_limit shortened them.  (Read at
+// run time by every wait, it cost 20 us of 1480 at 256 diagonals by 128 columns, N = 2^14.)
+template <bool SHORT>
+__device__ __forceinline__ unsigned tc_wait_limit(const TcGeom &g) {
+    return SHORT ? g.wait_limit : HE_WAIT_LIMIT;
+}
+
 // folds a unit's sums: the thread's 16 outputs are column 32 (warp % 4) + lane, rows 16 (fw / 4) + r
-template <int ND>
+template <int ND, bool SHORT>
 __device__ __forceinline__ bool tc_fold(const TcGeom &g, const TcTile &t, int kb, const TcLimb &lb, const ModConst &mc, uint64_t *pre, uint32_t tmem,
                                         uint32_t acc_full, uint32_t acc_empty, uint64_t *tr, uint32_t &slot_it) {
+    const unsigned limit = tc_wait_limit<SHORT>(g);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, part = (warp - 2) >> 2;
     const uint32_t lanes = (uint32_t)(warp & 3) << 21;  // the warp's quarter of the tensor-memory lanes
     int32_t dig[ND][16];
@@ -286,7 +294,7 @@ __device__ __forceinline__ bool tc_fold(const TcGeom &g, const TcTile &t, int kb
     bool ok = true;
     for (int m = 0; m < lb.n_mod && ok; ++m, ++slot_it) {
         const uint32_t slot = slot_it % TC_SLOTS;
-        ok = mbar_wait(acc_full + 8 * slot, (int)((slot_it / TC_SLOTS) & 1), ok, g.wait_limit);
+        ok = mbar_wait(acc_full + 8 * slot, (int)((slot_it / TC_SLOTS) & 1), ok, limit);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         float v[16];
         tmem_ld16(v, tmem + slot * TC_ROWS + (uint32_t)part * 16 + lanes);
@@ -342,6 +350,7 @@ __device__ __forceinline__ bool tc_fold(const TcGeom &g, const TcTile &t, int kb
 
 // Units: the slice's tiles by blocks of 128 columns; neighbouring CTAs take consecutive tiles (same limb,
 // orbit and nearly the same window), so the weights' blocks that each copies for itself come from L2.
+template <bool SHORT>
 __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __grid_constant__ TcGeom g, const __grid_constant__ CdiagTc tc,
                                                                      const TcLimb *__restrict__ limbs, const unsigned char *__restrict__ X, uint64_t *pre,
                                                                      const ModConst *__restrict__ mc, unsigned int *gave_up) {
@@ -374,6 +383,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(bars + 2 * TC_STAGES + 2 * TC_SLOTS);
     HE_GRID_WAIT();
     const int col_blocks = (g.K + TC_COLS - 1) / TC_COLS, units = g.tiles * col_blocks;
+    const unsigned limit = tc_wait_limit<SHORT>(g);
     bool ok = true;
     if (warp == 0) {
         if (lane == 0) {  // copies
@@ -388,7 +398,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
                 for (int m = 0; m < n_mod && ok; ++m)
                     for (int c = t.step0 / 4; c * 4 < t.step1 && ok; ++c, ++it) {
                         const uint32_t st = it % TC_STAGES;
-                        if (it >= TC_STAGES) ok = mbar_wait(empty + 8 * st, (int)((it / TC_STAGES - 1) & 1), ok, g.wait_limit);
+                        if (it >= TC_STAGES) ok = mbar_wait(empty + 8 * st, (int)((it / TC_STAGES - 1) & 1), ok, limit);
                         if (!ok) break;
                         const uint32_t bar = full + 8 * st, A = full_stage + st * TC_STAGE_BYTES;
                         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(TC_STAGE_BYTES) : "memory");
@@ -415,10 +425,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
             const int n_mod = limbs[t.u].n_mod;
             for (int m = 0; m < n_mod && ok; ++m, ++slot_it) {
                 const uint32_t slot = slot_it % TC_SLOTS, d = tmem + slot * TC_ROWS;
-                if (slot_it >= TC_SLOTS) ok = mbar_wait(acc_empty + 8 * slot, (int)((slot_it / TC_SLOTS - 1) & 1), ok, g.wait_limit);
+                if (slot_it >= TC_SLOTS) ok = mbar_wait(acc_empty + 8 * slot, (int)((slot_it / TC_SLOTS - 1) & 1), ok, limit);
                 for (int c = t.step0 / 4; c * 4 < t.step1 && ok; ++c, ++it) {
                     const uint32_t st = it % TC_STAGES;
-                    ok = mbar_wait(full + 8 * st, (int)((it / TC_STAGES) & 1), ok, g.wait_limit);
+                    ok = mbar_wait(full + 8 * st, (int)((it / TC_STAGES) & 1), ok, limit);
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t A = full_stage + st * TC_STAGE_BYTES;
@@ -444,8 +454,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) cdiag_tc_mma_kernel(const __gri
         for (int unit = blockIdx.x; unit < units && ok; unit += gridDim.x) {
             const TcTile t = tc_tile_of(g, g.first + unit % g.tiles);
             const TcLimb &lb = limbs[t.u];
-            if (lb.nd == 2) ok = tc_fold<2>(g, t, unit / g.tiles, lb, mc[t.u], pre, tmem, acc_full, acc_empty, tr, slot_it);
-            else ok = tc_fold<3>(g, t, unit / g.tiles, lb, mc[t.u], pre, tmem, acc_full, acc_empty, tr, slot_it);
+            if (lb.nd == 2) ok = tc_fold<2, SHORT>(g, t, unit / g.tiles, lb, mc[t.u], pre, tmem, acc_full, acc_empty, tr, slot_it);
+            else ok = tc_fold<3, SHORT>(g, t, unit / g.tiles, lb, mc[t.u], pre, tmem, acc_full, acc_empty, tr, slot_it);
         }
     }
     // every copy and product is complete: the tensor memory is free
@@ -603,10 +613,13 @@ void cdiag_tc_mac(he_ctx *ctx, const CdiagTc *tc, const he_ct *cts, int n_ct, in
             g.tiles = std::min(pass.slice, all - g.first);
             ctx->launches += 2;
             launch_k(cdiag_tc_residues_kernel, dim3((unsigned)g.tiles, (unsigned)g.chunks), TC_RES_THREADS, 0, ctx->stream, g, limbs, X);
-            launch_k(cdiag_tc_mma_kernel, std::min(ctx->sms, g.tiles * col_blocks), TC_THREADS, TC_SMEM, ctx->stream, g, *tc, limbs,
-                     (const unsigned char *)X, pre, (const ModConst *)ctx->d_mc, ctx->sh->gave_up);
+            launch_k(ctx->wait_limit < HE_WAIT_LIMIT ? cdiag_tc_mma_kernel<true> : cdiag_tc_mma_kernel<false>, std::min(ctx->sms, g.tiles * col_blocks),
+                     TC_THREADS, TC_SMEM, ctx->stream, g, *tc, limbs, (const unsigned char *)X, pre, (const ModConst *)ctx->d_mc, ctx->sh->gave_up);
         }
     }
 }
 
-void cdiag_tc_set_smem_limits() { cudaFuncSetAttribute(cdiag_tc_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM); }
+void cdiag_tc_set_smem_limits() {
+    cudaFuncSetAttribute(cdiag_tc_mma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+    cudaFuncSetAttribute(cdiag_tc_mma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+}
