@@ -66,7 +66,7 @@ struct TcLimb {
     int32_t nd;                 // signed 20-bit digits of a residue mod q: 2 below 2^40, else 3
     int32_t h[TC_MAX_MOD][3];   // (P/p_i) mod q, centred, as three signed 20-bit digits
     int32_t hk[3];              // P mod q likewise
-    int32_t init[3];            // cancels the bias of the integer form of y_i (see fold)
+    uint32_t init[3];           // of the digits' sums (tc_digit_init)
     int32_t inv[TC_MAX_MOD];    // (P/p_i)^-1 mod p_i
     uint64_t d40, d40_shoup;    // 2^40 mod q with its Shoup quotient
 };
@@ -283,7 +283,7 @@ __device__ __forceinline__ bool tc_fold(const TcGeom &g, const TcTile &t, int kb
     const unsigned limit = tc_wait_limit<SHORT>(g);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, part = (warp - 2) >> 2;
     const uint32_t lanes = (uint32_t)(warp & 3) << 21;  // the warp's quarter of the tensor-memory lanes
-    int32_t dig[ND][16];
+    uint32_t dig[ND][16];
     float frac[16];
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
@@ -309,9 +309,9 @@ __device__ __forceinline__ bool tc_fold(const TcGeom &g, const TcTile &t, int kb
         for (int r = 0; r < 16; ++r) {
             const float y = mod_centred(v[r], p, pinv);
             frac[r] = __fmaf_rn(y, pinv, frac[r]);
-            const int32_t yi = __float_as_int(__fadd_rn(y, TC_MAGIC));  // y + the bits of TC_MAGIC
+            const uint32_t yb = __float_as_uint(__fadd_rn(y, TC_MAGIC));
 #pragma unroll
-            for (int d = 0; d < ND; ++d) dig[d][r] += yi * h[d];
+            for (int d = 0; d < ND; ++d) dig[d][r] = tc_digit_add(dig[d][r], yb, h[d]);
         }
     }
     // V mod q = dig0 + dig1 2^20 + dig2 2^40 - round(frac) (P mod q)
@@ -319,10 +319,10 @@ __device__ __forceinline__ bool tc_fold(const TcGeom &g, const TcTile &t, int kb
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
         const int k = __float2int_rn(frac[r]);
-        const int64_t lo = (int64_t)dig[0][r] - (int64_t)k * lb.hk[0] + (((int64_t)dig[1][r] - (int64_t)k * lb.hk[1]) << 20);
+        const int64_t lo = (int64_t)(int32_t)dig[0][r] - (int64_t)k * lb.hk[0] + (((int64_t)(int32_t)dig[1][r] - (int64_t)k * lb.hk[1]) << 20);
         uint64_t v = reduce_signed(lo, q, mu);
         if constexpr (ND == 3) {
-            const int64_t h = (int64_t)dig[2][r] - (int64_t)k * lb.hk[2];
+            const int64_t h = (int64_t)(int32_t)dig[2][r] - (int64_t)k * lb.hk[2];
             const uint64_t hv = mul_shoup((uint64_t)(h < 0 ? -h : h), lb.d40, lb.d40_shoup, q);
             v = h < 0 ? sub_mod(v, hv, q) : add_mod(v, hv, q);
         }
@@ -536,7 +536,6 @@ int cdiag_tc_tables(he_ctx *ctx) {
         uint64_t pq = 1;
         for (int m = 0; m < lb.n_mod; ++m) pq = (uint64_t)((u128)pq * TC_MODULI[m] % q);
         digits20(lb.hk, pq, q, lb.nd);
-        const uint32_t bias = 0x4B400000u;  // the bits of 1.5 2^23
         for (int m = 0; m < lb.n_mod; ++m) {
             uint64_t h = 1, hp = 1;
             for (int j = 0; j < lb.n_mod; ++j)
@@ -546,7 +545,7 @@ int cdiag_tc_tables(he_ctx *ctx) {
                 }
             digits20(lb.h[m], h, q, lb.nd);
             lb.inv[m] = (int32_t)hinv_mod(hp, TC_MODULI[m]);
-            for (int d = 0; d < 3; ++d) lb.init[d] = (int32_t)((uint32_t)lb.init[d] - bias * (uint32_t)lb.h[m][d]);
+            for (int d = 0; d < 3; ++d) lb.init[d] = tc_digit_init(lb.init[d], lb.h[m][d]);
         }
         lb.d40 = (uint64_t)(((u128)1 << 40) % q);
         lb.d40_shoup = (uint64_t)(((u128)lb.d40 << 64) / q);

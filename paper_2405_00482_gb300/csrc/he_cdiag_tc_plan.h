@@ -50,6 +50,16 @@ inline TcPass tc_pass(int sms, int mods, int n_ct, int i0) {
     return p;
 }
 
+// A term y h of a digit's sum (h a signed digit, |h| <= 2^19; |y| <= 256), y as the bits of the float
+// 1.5 2^23 + y: TC_MAGIC_BITS + y.  The products and sums wrap mod 2^32; started at tc_digit_init, less
+// the bias of every term to come, a sum of at most TC_MAX_MOD terms ends as the exact value below 2^31.
+constexpr uint32_t TC_MAGIC_BITS = 0x4B400000u;
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline uint32_t tc_digit_add(uint32_t sum, uint32_t y_bits, int32_t h) { return sum + y_bits * (uint32_t)h; }
+inline uint32_t tc_digit_init(uint32_t init, int32_t h) { return init - TC_MAGIC_BITS * (uint32_t)h; }
+
 // operand scratch of a product of n_ct diagonals over `tiles` tiles: the largest slice of any pass.  A
 // short last pass has smaller tiles but more of them in a slice, and can need more than a full one (10
 // moduli, 152 SMs: 62 MB for 256 diagonals, 100 MB for the 44 left of 300).
