@@ -666,7 +666,7 @@ struct DecodeRas {
 };
 
 template <int CLG, int RL, int LOGN, class EPI>
-__global__ void decode_cl_kernel(const double *__restrict__ coeffs, double scale, const float4 *__restrict__ tw,
+__global__ void decode_cl_kernel(const double *coeffs, double scale, const float4 *__restrict__ tw,
                                  const float4 *__restrict__ twist, const int32_t *__restrict__ slot_pos, EPI epi, int logn_rt) {
     HE_GRID_LAUNCH();
     const int logn = LOGN ? LOGN : logn_rt;
@@ -702,7 +702,7 @@ __global__ void decode_cl_kernel(const double *__restrict__ coeffs, double scale
 // decrypt limb 0: m = c0 + c1 s (NTT), inverse NTT, centred, as doubles.  One CTA per
 // ciphertext, or (CL) one cluster per ciphertext with each CTA on a slice.
 template <bool CL, int LOGN = 0>
-__global__ void decrypt_kernel(const uint64_t *__restrict__ ct, int64_t ct_words, int nl, const uint64_t *__restrict__ sk_mont,
+__global__ void decrypt_kernel(const uint64_t *ct, int64_t ct_words, int nl, const uint64_t *__restrict__ sk_mont,
                                double *coeffs, const uint64_t *__restrict__ d_tw, const ModConst *__restrict__ mc, int logn_rt) {
     HE_GRID_LAUNCH();
     const int logn = LOGN ? LOGN : logn_rt;
@@ -873,7 +873,7 @@ __global__ void sample_ternary_kernel(uint64_t seed, int64_t *out, int logn) {
 // c0 = NTT(m + e) - c1 s: NTT(m) + NTT(e) = NTT(m + e) mod q, so the ciphertext equals that of
 // encoding m to a plaintext and encrypting it.
 template <int LOGN = 0>
-__global__ void __launch_bounds__(512) encrypt_ntt_cl_kernel(const int64_t *__restrict__ m_int, int nl, uint64_t seed, uint64_t nonce,
+__global__ void __launch_bounds__(512) encrypt_ntt_cl_kernel(const int64_t *m_int, int nl, uint64_t seed, uint64_t nonce,
                                                              const uint64_t *nonce_dev, Cdt cdt, uint64_t *ct, const uint64_t *__restrict__ d_tw,
                                                              const ModConst *__restrict__ mc, int logn_rt) {
     HE_GRID_LAUNCH();

@@ -409,7 +409,9 @@ int ptmat_bind_keys(he_ctx *ctx, he_ptmat *pm);
 // The two halves, for kernels that start loads before the wait.  Those loads may read only the
 // context's tables written at its creation (which synchronises), never data of an earlier launch:
 // with every kernel releasing its successor on entry, a kernel's pre-wait code can run while
-// kernels two or more launches back are still running.
+// kernels two or more launches back are still running.  A pointer that earlier launches write through
+// carries no __restrict__ in such a kernel: its loads would count as invariant, which the compiler may
+// move above the wait (one was, in the one-launch product and rescale).
 #define HE_GRID_LAUNCH() asm volatile("griddepcontrol.launch_dependents;" ::: "memory")
 #define HE_GRID_WAIT() asm volatile("griddepcontrol.wait;" ::: "memory")
 

@@ -284,7 +284,7 @@ __device__ __forceinline__ void modup_cl_fused_body(const uint64_t *__restrict__
 }
 
 template <int LOGN = 0>
-__global__ void modup_cl_fused_kernel(const uint64_t *__restrict__ c1_ntt, uint64_t *D, ModUpConst mu, const uint64_t *__restrict__ d_tw,
+__global__ void modup_cl_fused_kernel(const uint64_t *c1_ntt, uint64_t *D, ModUpConst mu, const uint64_t *__restrict__ d_tw,
                                       const ModConst *__restrict__ mc, int logn_rt) {
     HE_GRID_LAUNCH();
     const int logn = LOGN ? LOGN : logn_rt;
@@ -459,9 +459,8 @@ __device__ __forceinline__ void moddown_rescale_intt_body(const uint64_t *__rest
 }
 
 template <int LOGN = 0>
-__global__ void moddown_rescale_intt_kernel(const uint64_t *__restrict__ x, int ext, ModDownConst md, const uint64_t *__restrict__ add0,
-                                            const uint64_t *__restrict__ add1, uint64_t *tmp, const uint64_t *__restrict__ d_tw,
-                                            const ModConst *__restrict__ mc, int logn_rt) {
+__global__ void moddown_rescale_intt_kernel(const uint64_t *x, int ext, ModDownConst md, const uint64_t *add0, const uint64_t *add1,
+                                            uint64_t *tmp, const uint64_t *__restrict__ d_tw, const ModConst *__restrict__ mc, int logn_rt) {
     HE_GRID_LAUNCH();
     const int logn = LOGN ? LOGN : logn_rt;
     int item, off, len;
@@ -526,9 +525,8 @@ __device__ __forceinline__ void moddown_rescale_ntt_body(const uint64_t *__restr
 }
 
 template <int LOGN = 0>
-__global__ void moddown_rescale_ntt_kernel(const uint64_t *__restrict__ x, int ext, ModDownConst md, RescaleConst rc,
-                                           const uint64_t *__restrict__ add0, const uint64_t *__restrict__ add1, const uint64_t *__restrict__ tmp,
-                                           uint64_t *out, const uint64_t *__restrict__ d_tw, const ModConst *__restrict__ mc, int logn_rt) {
+__global__ void moddown_rescale_ntt_kernel(const uint64_t *x, int ext, ModDownConst md, RescaleConst rc, const uint64_t *add0,
+                                           const uint64_t *add1, const uint64_t *tmp, uint64_t *out, const uint64_t *__restrict__ d_tw, const ModConst *__restrict__ mc, int logn_rt) {
     HE_GRID_LAUNCH();
     const int logn = LOGN ? LOGN : logn_rt;
     int item, off, len;
@@ -1437,9 +1435,8 @@ __device__ __forceinline__ void stage_tables(MMTables &tb, const uint64_t *const
 // fused = the plaintext block's fused key tables [m'-1][NDIG][2][ext][N]
 template <int NDIG, int VEC, int G, int S, bool GA, bool FK = false>
 __global__ void __launch_bounds__(MM_THREADS, VEC == 2 ? 2 : 3) matmult_loop_kernel(
-    const uint64_t *__restrict__ ct, const uint64_t *__restrict__ D, const uint64_t *__restrict__ pts,
-    const uint64_t *const *__restrict__ keys, const uint32_t *__restrict__ galois, int m_prime, int ndig_rt, int ext, int nq, int L,
-    int LK, uint64_t *acc, uint64_t *cacc, int accumulate, const ModConst *__restrict__ mc, int logn, const uint64_t *__restrict__ fused,
+    const uint64_t *ct, const uint64_t *D, const uint64_t *pts, const uint64_t *const *keys, const uint32_t *galois, int m_prime, int ndig_rt, int ext,
+    int nq, int L, int LK, uint64_t *acc, uint64_t *cacc, int accumulate, const ModConst *__restrict__ mc, int logn, const uint64_t *fused,
     int tables_ready) {
     HE_GRID_LAUNCH();
     __shared__ uint64_t red[G * 3 * VEC * (MM_THREADS / G)];
