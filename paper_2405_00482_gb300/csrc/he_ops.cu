@@ -1496,7 +1496,7 @@ __global__ void __launch_bounds__(256) fuse_keys_kernel(const uint64_t *__restri
 // PM the Montgomery form of P mod q_u: a term P x of the accumulator becomes exactly x in ModDown, so
 // the c0 part needs no accumulator of its own, nor does step 0, which is added as P c0 pt and P c1 pt.
 // Sums mod q of the same terms, so the rescaled ciphertexts are those of matmult_loop_kernel.
-// The tile is that of loop variant 5 (16-byte copies into private stages, gathers too).  Two rows are
+// The tile is that of loop variant MMR_VARIANT (16-byte copies into private stages, gathers too).  Two rows are
 // what 128 registers hold (two CTAs of 7-8 warps per multiprocessor); a step of two row blocks costs 11
 // 128-bit multiply-adds and 2 reductions instead of 18 and 4.  N = 2^13, 4 extended limbs, 3 digits, 511
 // rotations: 243 us for two row blocks (1.07 GB read, 4.4 TB/s, 46% of the issue slots: bound by the
@@ -1697,6 +1697,10 @@ constexpr MMShape kMMShapes[] = {{2, 4, 0, false}, {1, 4, 0, false}, {1, 8, 0, f
                                  {2, 4, 3, false}, {2, 4, 2, true},  {1, 4, 2, true},  {1, 8, 2, true}};
 constexpr int kMMVariants = (int)(sizeof(kMMShapes) / sizeof(kMMShapes[0]));
 static_assert(kMMVariants <= HE_MM_MAX_VARIANTS, "variant table");
+constexpr int MMR_VARIANT = 5;  // the loop variant whose tile, and so its split into blocks, the rows form has
+static_assert(kMMShapes[MMR_VARIANT].vec == MMR_VEC && kMMShapes[MMR_VARIANT].grp == MMR_G && kMMShapes[MMR_VARIANT].stages == MMR_S &&
+                  kMMShapes[MMR_VARIANT].ga,
+              "tile of matmult_rows_kernel");
 
 int mm_variant_count() { return kMMVariants; }
 int mm_variant_tile(int v) { return (MM_THREADS / kMMShapes[v].grp) * kMMShapes[v].vec; }
@@ -2078,7 +2082,7 @@ void launch_matmult_rows(he_ctx *ctx, const he_ptmat *pm, int r, int c, const ui
     const ModUpConst &mu = ctx->modup[pm->level];
     const he_plan &p = pm->plan;
     const int64_t block = p.m_prime * pm->ext * ctx->n, total = (int64_t)mu.ext * (ctx->n / MMR_VEC);
-    const int lanes = mm_block_lanes(5, total, ctx->sms);  // variant 5 has the same lanes and groups
+    const int lanes = mm_block_lanes(MMR_VARIANT, total, ctx->sms);
     MMRowsConst rc{};
     for (int j = 0; j <= pm->level; ++j) {
         const uint64_t q = ctx->primes[j];
