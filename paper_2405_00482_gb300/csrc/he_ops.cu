@@ -816,14 +816,15 @@ __device__ __forceinline__ uint64_t fold_wide(u128 t, uint64_t q, uint64_t qinv,
     return redc(reduce_barrett((uint64_t)(t >> 64), q, mu), (uint64_t)t, q, qinv);
 }
 
+// (an ordinary load, not __ldg: what earlier launches wrote must not be read above the dependent-launch wait)
 template <int VEC>
 __device__ __forceinline__ void ldv(const uint64_t *p, uint64_t (&o)[VEC]) {
     if constexpr (VEC == 2) {
-        const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2 *>(p));
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(p);
         o[0] = t.x;
         o[1] = t.y;
     } else {
-        o[0] = __ldg(p);
+        o[0] = *p;
     }
 }
 // gather of VEC values at the automorphism image of k..k+VEC-1 (src of k given)
