@@ -546,8 +546,6 @@ __global__ void encode_pair_cl_kernel(SRC src, int count, double scale, const fl
     cl.sync();  // the other CTAs read this one's shared memory until here
 }
 
-// cluster per polynomial: each CTA loads the coefficients whose bit-reversed positions it holds;
-// the slot values are read from the owning CTAs
 // What the decode writes once the slot values are in the cluster's shared memory.  DecodeSlots:
 // slot j of plaintext `item` to out[item][j].  DecodeRas: the lazy rotate-and-sum of the rows of
 // row block `item` (Sec. 4.3), y[row] = sum over s < nb/m' of slot[b nb + t + s m'] (minus the
@@ -555,12 +553,6 @@ __global__ void encode_pair_cl_kernel(SRC src, int count, double scale, const fl
 // slot values, so the same doubles without the slot array.
 // Each epilogue's slot positions of its first two iterations are read by prefetch() before the
 // kernel waits for its predecessor.
-// the ciphertexts of one fused decryption
-constexpr int HE_DECRYPT_MAX = 16;
-struct DecryptSrc {
-    const uint64_t *ct[HE_DECRYPT_MAX];
-    int32_t nl[HE_DECRYPT_MAX];  // limbs of each component
-};
 struct EpiPre {
     int pos[2];
 };
@@ -665,6 +657,8 @@ struct DecodeRas {
     }
 };
 
+// cluster per polynomial: each CTA loads the coefficients whose bit-reversed positions it holds;
+// the slot values are read from the owning CTAs
 template <int CLG, int RL, int LOGN, class EPI>
 __global__ void decode_cl_kernel(const double *coeffs, double scale, const float4 *__restrict__ tw,
                                  const float4 *__restrict__ twist, const int32_t *__restrict__ slot_pos, EPI epi, int logn_rt) {
@@ -725,6 +719,12 @@ __global__ void decrypt_kernel(const uint64_t *ct, int64_t ct_words, int nl, con
     }
 }
 
+// the ciphertexts of one fused decryption
+constexpr int HE_DECRYPT_MAX = 16;
+struct DecryptSrc {
+    const uint64_t *ct[HE_DECRYPT_MAX];
+    int32_t nl[HE_DECRYPT_MAX];  // limbs of each component
+};
 // decrypt_kernel<true> and decode_cl_kernel in one launch, a cluster per ciphertext: each CTA sends the
 // centred coefficients of its slice straight to their bit-reversed places in the cluster's shared
 // memory (stores, which nothing waits for; gathering them instead, with 4-way bank conflicts on loads

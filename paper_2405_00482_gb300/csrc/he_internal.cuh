@@ -525,10 +525,12 @@ bool launch_encode_matrix(he_ctx *ctx, const he_plan &p, const double *X, int tr
 bool launch_encode_vector(he_ctx *ctx, const he_plan &p, const double *y, int count, double scale, int64_t *coeffs);
 void launch_decode(he_ctx *ctx, const double *coeffs, int count, double scale, double *slots);
 void launch_decrypt_coeffs(he_ctx *ctx, const uint64_t *ct, int level, int count, double *coeffs, uint64_t *tmp);
+// decryption and decode of one ciphertext in one launch, and of the row blocks' ciphertexts with the lazy
+// rotate-and-sum of the plan, into y [m]; false (nothing launched) where that form does not apply
+bool launch_decrypt_slots(he_ctx *ctx, const he_ct *ct, double *slots);
+bool launch_decrypt_ras(he_ctx *ctx, const he_plan &p, const he_ct *cts, int count, const double *mask, double *y);
 // decode of `count` decrypted coefficient vectors (the row blocks' output ciphertexts) with the lazy
 // rotate-and-sum of the plan in the same launch, into y [m]; false where that form does not apply
-bool launch_decrypt_slots(he_ctx *ctx, const he_ct *ct, double *slots);  // decryption and decode in one launch, if they fit
-bool launch_decrypt_ras(he_ctx *ctx, const he_plan &p, const he_ct *cts, int count, const double *mask, double *y);
 bool launch_decode_ras(he_ctx *ctx, const he_plan &p, const double *coeffs, int count, double scale, const double *mask, double *y);
 // he_encrypt's five steps as one cluster launch per limb (false: that form does not apply); with
 // m_int (integer coefficients, pt null) the plaintext is encoded into the same launch

@@ -172,18 +172,18 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) ntt2_cols_kernel(const void *
     uint64_t *dst = out + g * out_gs + (int64_t)l * N;
     if constexpr (I64) {  // int64 coefficients, shared by the limbs of group g, reduced mod q
         const int64_t *src = static_cast<const int64_t *>(in_v) + g * in_gs;
-        ntt2_fwd_cols<LOGN>(sm, 
-            [=](int64_t x) { return src[x]; },
+        ntt2_fwd_cols<LOGN>(
+            sm, [=](int64_t x) { return src[x]; },
             [=](uint64_t w) {
                 const uint64_t v = lift_signed((int64_t)w, q, lift, mu);
                 return to_mont ? mul_shoup_lazy(v, r1, r1s, q) : v;
             },
-            dst, c0,
-                            TwGlobal{twiddles(d_tw, p, 0, LOGN)}, q);
+            dst, c0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, q);
     } else {
         const uint64_t *src = static_cast<const uint64_t *>(in_v) + g * in_gs + (int64_t)l * N;
-        ntt2_fwd_cols<LOGN>(sm, [=](int64_t x) { return src[x]; }, [=](uint64_t v) { return to_mont ? mul_shoup_lazy(v, r1, r1s, q) : v; }, dst, c0,
-                            TwGlobal{twiddles(d_tw, p, 0, LOGN)}, q);
+        ntt2_fwd_cols<LOGN>(
+            sm, [=](int64_t x) { return src[x]; }, [=](uint64_t v) { return to_mont ? mul_shoup_lazy(v, r1, r1s, q) : v; }, dst, c0,
+            TwGlobal{twiddles(d_tw, p, 0, LOGN)}, q);
     }
 }
 
@@ -198,7 +198,9 @@ __global__ void __launch_bounds__(NTT2_THREADS, 8) ntt2_cols_tab_kernel(const in
     const int g = poly / map.n, l = poly % map.n, p = map.prime[l];
     const uint64_t q = mc[p].q, lift = mc[p].lift, mu = mc[p].mu;
     const int64_t *src = in + (int64_t)g * N;
-    ntt2_fwd_cols<LOGN>(sm, [=](int64_t x) { return src[x]; }, [=](uint64_t v) { return lift_signed((int64_t)v, q, lift, mu); }, outs.p[g] + (int64_t)l * N, c0, TwGlobal{twiddles(d_tw, p, 0, LOGN)}, q);
+    ntt2_fwd_cols<LOGN>(
+        sm, [=](int64_t x) { return src[x]; }, [=](uint64_t v) { return lift_signed((int64_t)v, q, lift, mu); }, outs.p[g] + (int64_t)l * N, c0,
+        TwGlobal{twiddles(d_tw, p, 0, LOGN)}, q);
 }
 template <int LOGN>
 __global__ void __launch_bounds__(NTT2_THREADS, 8) ntt2_rows_tab_kernel(const __grid_constant__ OutPtrs outs, LimbMap map, const uint64_t *__restrict__ d_tw,

@@ -378,8 +378,9 @@ __host__ __device__ constexpr int ntt2_rows_smem_words(int lb) { return NTT2_TR 
 __host__ __device__ constexpr int ntt2_frows_smem_words(int lb) { return NTT2_TR * (1 << lb) + NTT2_TR * (1 << lb) / 32; }
 __device__ __forceinline__ int ntt2_at(int m) { return m + (m >> 3); }
 
-// forward stages 0-5 of columns c0 .. c0 + NTT2_TC - 1 of one limb-poly, inputs below 4q (or lift_signed's),; writes the stage-5 values to dst[x]
-// input of element x from the word at x: prep(load(x)), all eight loads of a thread before the first prep
+// forward stages 0-5 of columns c0 .. c0 + NTT2_TC - 1 of one limb-poly; writes the stage-5 values to
+// dst[x].  Element x's input is prep(load(x)), below 4q (or lift_signed's), all eight loads of a thread
+// before the first prep
 template <int LOGN, class LOAD, class PREP>
 __device__ __forceinline__ void ntt2_fwd_cols(uint64_t *sm, LOAD load, PREP prep, uint64_t *dst, int c0, TwGlobal tw, uint64_t q) {
     constexpr int C = (1 << LOGN) >> 6, PAD = NTT2_TC + 1;

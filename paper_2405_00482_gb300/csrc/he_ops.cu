@@ -827,7 +827,7 @@ __device__ __forceinline__ void ldv(const uint64_t *p, uint64_t (&o)[VEC]) {
         o[0] = *p;
     }
 }
-// gather of VEC values at the automorphism image of k..k+VEC-1 (src of k given)
+// the same with an L2 replacement policy
 template <int VEC>
 __device__ __forceinline__ void ldv(const uint64_t *p, uint64_t (&o)[VEC], uint64_t policy) {
     if constexpr (VEC == 2)
@@ -835,6 +835,7 @@ __device__ __forceinline__ void ldv(const uint64_t *p, uint64_t (&o)[VEC], uint6
     else
         asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u64 %0, [%1], %2;" : "=l"(o[0]) : "l"(p), "l"(policy));
 }
+// gather of VEC values at the automorphism image of k..k+VEC-1 (src of k given)
 template <int VEC>
 __device__ __forceinline__ void gatherv(const uint64_t *base, uint32_t src, uint64_t (&o)[VEC]) {
     if constexpr (VEC == 2) {
