@@ -421,9 +421,9 @@ void he_server_free(he_server *s);
  * with the plaintext rotation done as the automorphism X -> X^(5^i) of w_k's plaintext (no
  * key switching: "eliminate all O4").  After decryption, he_cdiag_decode turns the K slot
  * vectors (device [K][N/2]) into Z = A W (device, m x K row-major), summing the n/m slot
- * groups when m < n (lazy rotate-and-sum, Sec. 4.3).  n_ct <= 1024 per call.  Products of at
- * least 20 ciphertexts by 8 columns run on the tensor cores, exactly (the same residues), in kernels with
- * bounded waits (HE_ETIMEOUT: see he_synchronize). */
+ * groups when m < n (lazy rotate-and-sum, Sec. 4.3).  n_ct <= 1024 per call.  Products of about
+ * 20 and more ciphertexts by 8 and more columns run on the tensor cores, exactly (the same residues), in
+ * kernels with bounded waits (HE_ETIMEOUT: see he_synchronize). */
 typedef struct he_cdmat he_cdmat;
 int he_cdiag_encode_weights(he_ctx *ctx, const double *W, int64_t n, int64_t K, int level, he_cdmat **out);
 void he_cdmat_free(he_cdmat *W);

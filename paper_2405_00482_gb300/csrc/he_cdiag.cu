@@ -22,16 +22,14 @@
 #define CD_MAX_IN 1024 // ciphertexts per launch (kernel-parameter table)
 #define CD_MAX_OUT 512 // outputs per rescale launch
 // The tensor cores (rings of 2^12 to 2^14, primes below 2^60: cdiag_tc_supported) take products of at
-// least 20 diagonals by at least 8 columns.  Their time hardly depends on the diagonals up to a window of
-// 64, that of the integer form is proportional to them and the same for 1 as for 128 columns.  The whole
-// call, tensor cores / integer form, in us for 2, 8, 16, 20, 24, 32 and 64 diagonals:
+// least 8 columns and tc_min_diags diagonals (8 to 25 on the rings in use).  The whole call, tensor cores /
+// integer form, in us for 2, 8, 16, 20, 24, 32 and 64 diagonals:
 //   N = 2^12,    8 columns, n =   64:    60/41   62/52   63/67   63/74   64/82   65/97   68/154
 //   N = 2^13,   16 columns, n =  256:   152/63  157/94 157/135 161/154 162/175 164/217  178/394
 //   N = 2^13,    8 columns, n = 4096:  186/82 189/112 194/155 199/173 204/194 214/235  268/400
 //   N = 2^14,    8 columns, n =   64: 476/162 488/302 497/505 506/601 515/695 525/890 558/1660
 //   N = 2^14,  128 columns, n =  256: 844/587 863/748 877/970 881/1078 882/1186 891/1406 928/2279
 #define CD_TC_MIN_COLS 8
-#define CD_TC_MIN_DIAGS 20
 
 struct he_cdmat {
     he_ctx *ctx;
@@ -40,6 +38,7 @@ struct he_cdmat {
     double scale;
     uint64_t *pt;  // [level+1][N][K], NTT + Montgomery form
     CdiagTc tc;    // the tensor-core form besides (he_cdiag_tc.cu), where products may take it
+    int tc_min;    // diagonals from which they do
 };
 
 namespace {
@@ -277,7 +276,8 @@ int he_cdiag_encode_weights(he_ctx *ctx, const double *W, int64_t n, int64_t K, 
     launch_k(transpose_cols_kernel, blocks_for(K * nl * N), 256, 0, ctx->stream, cols, cm->pt, (int)K, (int)nl, ctx->log_n);
     bool ok = cudaGetLastError() == cudaSuccess;
     // the weights' residues pad the columns to 128: without memory for them the integer form serves
-    if (K >= CD_TC_MIN_COLS && n >= CD_TC_MIN_DIAGS && cdiag_tc_supported(ctx, level)) {
+    cm->tc_min = tc_min_diags(ctx->primes.data(), (int)nl, n, K);
+    if (K >= CD_TC_MIN_COLS && n >= cm->tc_min && cdiag_tc_supported(ctx, level)) {
         const bool prepared = cdiag_tc_prepare(ctx, &cm->tc, n, K, level, cols);
         ok = ok && (cudaGetLastError() == cudaSuccess || !prepared);
     }
@@ -335,7 +335,7 @@ int he_cdiag_matmult(he_ctx *ctx, const he_cdmat *W, const he_ct *cts, int n_ct,
     const int64_t K = W->K, N = ctx->n;
     for (int64_t k = 0; k < K; ++k)
         if (!outs[k].data) return HE_EINVAL;
-    bool tc = W->tc.wt && n_ct >= CD_TC_MIN_DIAGS;
+    bool tc = W->tc.wt && n_ct >= W->tc_min;
     if (tc && wait_gave_up(ctx)) return HE_ETIMEOUT;
     const size_t w_pre = (size_t)K * 2 * nl * N, w_last = (size_t)K * 2 * N;
     // the integer form where the operands' scratch cannot be had: no memory, or a stream under capture

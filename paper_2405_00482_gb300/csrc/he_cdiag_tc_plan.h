@@ -28,6 +28,30 @@ inline int tc_moduli(uint64_t q) {
     return 0;
 }
 
+// Diagonals from which the tensor cores take a product of n weight rows by K columns (8 and more) sooner
+// than the integer form.  The integer form's time is proportional to the diagonals and the blocks of 128
+// columns; that of the tensor cores, up to a window of 64 diagonals, to the moduli (three-digit limbs
+// cost 1.6 of the others in conversion and reconstruction), to the window's chunks (one for n <= 32,
+// more as a window of n = 64 and more begins anywhere in a chunk) and, for the longest periods, to the
+// weights, which outgrow L2.  More columns fill the same instructions; columns that are no multiple of 8
+// slow the integer form's loads.  The factors are fitted to both forms' times over N = 2^12 (2 limbs), 2^13
+// (3) and 2^14 (3 and 7), 8 to 200 columns, 8 to 8192 rows and 4 to 32 diagonals: the chosen form takes
+// 1.004 times the faster one's time on average, 1.16 at worst.  At N = 2^14, 7 limbs, in us, tensor cores /
+// integer form for 8, 12, 16, 20 and 24 diagonals, then the line:
+//     8 columns, n =   16: 437/305 437/401 440/503                    14
+//     8 columns, n =  256: 509/296 517/391 522/493 526/593 527/690    18
+//     8 columns, n = 8192: 542/296 552/392 567/495 585/593 611/691    20
+//    30 columns, n =  256: 591/429 600/544 605/664 608/780            15
+//   128 columns, n =  256: 863/749 871/855 876/969 881/1077 883/1184  15
+inline int tc_min_diags(const uint64_t *primes, int nl, int64_t n, int64_t K) {
+    int64_t cost = 0;  // in fifths of a two-digit limb's modulus
+    for (int u = 0; u < nl; ++u) cost += tc_moduli(primes[u]) * (primes[u] >> 40 ? 8 : 5);
+    const int rows = n <= 32 ? 7 : n <= 64 ? 8 : n <= 2048 ? 9 : 10;  // sixths of a diagonal per modulus
+    const int cols = (K < 96 ? 5 : K <= 128 ? 4 : 3) * (K % 8 ? 4 : 5);  // twenty-fifths
+    const int64_t den = 5 * 6 * 25 * (int64_t)nl;
+    return (int)((cost * rows * cols + den - 1) / den);
+}
+
 // chunks of the longest window of cnt diagonals: its start is rounded down to a whole chunk from the
 // tile's first block, a multiple of the span (at most 32) of its blocks: 64 - span, span - 1 and the
 // diagonals

@@ -34,6 +34,7 @@ extern "C" int32_t digit_sum(int n, const float *y, const int32_t *h) {
     }
     return (int32_t)sum;
 }
+extern "C" int min_diags(const uint64_t *primes, int nl, int64_t n, int64_t k) { return tc_min_diags(primes, nl, n, k); }
 extern "C" int moduli(uint64_t q) { return tc_moduli(q); }
 """
 
@@ -80,3 +81,14 @@ def test_digit_sums_are_exact_without_signed_overflow(lib):
         want = sum(a * b for a, b in zip(y, h))
         assert abs(want) < 1 << 31
         assert lib.digit_sum(n, (ctypes.c_float * n)(*y), (ctypes.c_int32 * n)(*h)) == want
+
+
+@pytest.mark.parametrize("bits,n,cols,want", [([40, 20], 64, 8, 11), ([40, 20], 2048, 128, 10), ([60, 40, 40], 32, 8, 18), ([60, 40, 40], 64, 8, 20),
+                                              ([60, 40, 40], 4096, 8, 25), ([60] + [40] * 6, 16, 8, 14), ([60] + [40] * 6, 64, 8, 16),
+                                              ([60] + [40] * 6, 256, 128, 15), ([60] + [40] * 6, 8192, 8, 20), ([60] + [40] * 6, 8192, 200, 12),
+                                              ([60] + [40] * 6, 256, 30, 15), ([60] + [40] * 6, 256, 101, 12)])
+def test_line_between_the_forms(lib, bits, n, cols, want):
+    """tc_min_diags for the parameter sets' prime sizes (primes just below the powers of two)."""
+    primes = (ctypes.c_uint64 * len(bits))(*[(1 << b) - 87 for b in bits])
+    lib.min_diags.argtypes = [ctypes.POINTER(ctypes.c_uint64), ctypes.c_int, ctypes.c_int64, ctypes.c_int64]
+    assert lib.min_diags(primes, len(bits), n, cols) == want

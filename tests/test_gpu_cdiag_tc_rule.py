@@ -1,4 +1,4 @@
-"""Which form a ciphertext-diagonal product takes: the integer form below 20 diagonals, and where the
+"""Which form a ciphertext-diagonal product takes: the integer form for few diagonals, and where the
 tensor cores' scratch cannot grow (a stream under capture); the same residues either way."""
 import gc
 
@@ -30,7 +30,7 @@ def _narrow(he, ctx, W, cts):
     return outs
 
 
-@pytest.mark.parametrize("n,count,tensor", [(64, 1, False), (64, 19, False), (64, 20, True), (32, 32, True), (4096, 19, False), (16, 16, False)])
+@pytest.mark.parametrize("n,count,tensor", [(64, 1, False), (64, 19, False), (64, 20, True), (32, 32, True), (4096, 24, False), (4096, 25, True), (16, 16, False)])
 def test_by_diagonals(n, count, tensor):
     import torch
 
