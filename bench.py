@@ -828,8 +828,8 @@ def run_batched(ctx, he, inputs, P, args, flush, world, dev):
     batch_roof = {"bound": "alu (integer multiply issue)", "hbm_achieved": round(alg / b_s / 1e9, 1), "hbm_peak": peak, "unit": "GB/s",
                   "hbm_frac": round(alg / b_s / 1e9 / peak, 4), "alg_bytes_per_batch": alg,
                   "counted": "plaintexts of every job (m' x (l+1+K) limbs) + Galois keys once + input and output ciphertexts",
-                  "note": "the loop kernel is about 95% of the batch; ncu: ~220 thread instructions per (rotation, limb, coefficient) on 60-bit primes, "
-                          "issue active ~50%"}
+                  "note": "the loop kernel is about 95% of the batch; ncu: 211 thread instructions per (rotation, limb, coefficient) over 60- and 40-bit primes, "
+                          "multiplier pipe 71%, issue active 53%"}
     return {"value": round(whole_job_rate(64 * args.steps, world, sb), 1), "unit": "MatMult/s",
             "plain_same_jobs": round(whole_job_rate(64 * args.steps, world, sp), 1), "speedup_vs_plain": round(sp / sb, 3),
             "plain_same_jobs_fused_tables": sum(1 for f in fused_state if f == 1),

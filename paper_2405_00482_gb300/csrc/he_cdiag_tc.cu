@@ -36,13 +36,15 @@
 // fold each modulus' sums from tensor memory (8 slots of 64 columns) into the reconstruction's
 // registers, all three running ahead of each other by their rings.  Every CTA copies all of the weights'
 // blocks for itself: the copies are not what it waits for (halves shared within a pair of CTAs took the
-// same time, 1.50 against 1.49 ms for the whole call).  The results go through shared memory so that half a warp stores 16
-// rows of one column (stored from the registers, one column per lane, they took 8.5 of a slice's 40 us).
+// same time, 1.50 against 1.49 ms for the whole call).  The results go through shared memory so that half a
+// warp stores 16 rows of one column (stored from the registers, one column per lane, they took 8.5 of a
+// slice's 40 us).
 //
 // 4096 x 256 activations (256 diagonals) by 128 columns at N = 2^14, 7 limbs: 7.5 G modular
-// multiply-adds in 0.44 ms (residues: float and integer issue, 65% active) and 0.63 ms (products:
-// the issue of short tensor instructions, about 100 cycles each, and the start and end of each slice),
-// against 6.26 ms for the 64-bit integer form (cdiag_mac_kernel), which the multiplier pipe bounds.
+// multiply-adds in 0.43 ms (residues: float and integer issue, 68% active) and 0.63 ms (products: short
+// tensor instructions about 100 cycles apart, tensor pipe 12% active, and the start and end of each slice),
+// against 6.26 ms for the 64-bit integer form (cdiag_mac_kernel), whose multiply-adds take 22 integer
+// instructions each.
 
 #include <algorithm>
 #include <vector>
